@@ -389,6 +389,9 @@ lbm_status lbm_create(const lbm_domain* domain, const lbm_cylinder* cyl, const l
     phys.ka2 = split(k * P.a);
     phys.k32 = split(k / 3.0);
   }
+  phys.rTc = 1.0 / ph.Tc;
+  phys.rdr = 1.0 / (ph.rho_l - ph.rho_v);
+  phys.rGc = 1.0 / (ph.G * (1.0 / 3.0));
   phys.dpdT_c1 = (float)(eos.kappa * (1.0 + eos.kappa));
   phys.dpdT_c2 = (float)(eos.kappa * eos.kappa / eos.Tc);
   {
@@ -546,6 +549,10 @@ lbm_status lbm_create(const lbm_domain* domain, const lbm_cylinder* cyl, const l
   d.rho = dalloc(c, 3 * N * es);
   d.ux = d.rho ? static_cast<char*>(d.rho) + N * es : nullptr;
   d.uy = d.rho ? static_cast<char*>(d.rho) + 2 * N * es : nullptr;
+  // the FP64 energy pass hands lambda, T1 and the frozen parts of the equation between its kernels
+  const bool en64 = c->f64 && P.energy;
+  d.lam = en64 ? dalloc(c, 8 * N * es) : nullptr;
+  d.en64 = d.lam ? static_cast<char*>(d.lam) + N * es : nullptr;
   d.side[0] = dalloc(c, 3 * (size_t)g.ny * es);
   d.side[1] = dalloc(c, 3 * (size_t)g.ny * es);
   d.partial = static_cast<double*>(dalloc(c, sizeof(double) * lbm::energy_blocks(g.nx, g.ny)));
@@ -580,7 +587,7 @@ lbm_status lbm_create(const lbm_domain* domain, const lbm_cylinder* cyl, const l
   g.wall_n = dwn;
   // staging planes for host I/O: a whole state (9 populations, T) and the outlet rows in one copy
   d.stage = static_cast<double*>(dalloc(c, sizeof(double) * ((size_t)g.nx * g.ny * 10 + 3 * (size_t)g.ny)));
-  if (!d.f[0] || !d.f[1] || !d.T[0] || !d.T[1] || !d.psi || !d.psi_next || !d.rho || !d.ux || !d.uy || !d.side[0] ||
+  if ((en64 && !d.lam) || !d.f[0] || !d.f[1] || !d.T[0] || !d.T[1] || !d.psi || !d.psi_next || !d.rho || !d.ux || !d.uy || !d.side[0] ||
       !d.side[1] || !d.partial || !d.counter || !dmask || !dbn || !dbv || !d.hf || !d.status || !d.stage ||
       !dwidx || !dwq || !dwn) {
     dfree_all(c);

@@ -56,6 +56,7 @@ struct Phys {
   F2 kR2, ka2, k32;  // k R, k a, k / 3 with k = 2 / (G cs^2): the double-float psi's folded constants
   F2 K12;            // 1 + kappa (the same)
   float dpdT_c1, dpdT_c2;  // kappa (1 + kappa) and kappa^2 / Tc: (dp/dT)_rho of the FP32 energy pass
+  double rTc, rdr, rGc;  // 1 / T_c, 1 / (rho_l - rho_v), 1 / (G cs^2): reciprocals of the FP64 divisors
   float pop_shift[9];  // shifted FP16 storage keeps f_i - w_i rho_l; these are w_i rho_l
 };
 
@@ -82,6 +83,8 @@ struct Dev {
   void* psi;         // pseudopotential of the current step
   void* psi_next;    // pseudopotential of the next step, when the energy pass computed it
   void* t1_out;      // if set, the energy pass also stores its stage-1 temperature T1 here
+  void* lam;         // lambda(rho) of the last collision (FP64 energy pass)
+  void* en64;        // work planes of the FP64 energy pass: T1 and six frozen parts
   void* rho;         // density of the last collision
   void* ux;          // velocity of the last collision
   void* uy;

@@ -89,6 +89,16 @@ __device__ __forceinline__ float fdiv<float>(float a, float b) {
   return __fdividef(a, b);
 }
 
+// a / b with rb = 1 / b rounded to nearest.  FP64: q = a rb corrected by its exact remainder, which is
+// the correctly rounded quotient (P. Markstein, IBM J. Res. Dev. 34, 1990; N. Brisebarre, J.-M. Muller,
+// S. K. Raina, IEEE Trans. Comput. 53, 2004): 3 operations on the FP64 pipe instead of about 10 where
+// the divisor is a constant or used more than once.  FP32: a / b as fdiv.
+__device__ __forceinline__ double div_by(double a, double b, double rb) {
+  const double q = __dmul_rn(a, rb);
+  return __fma_rn(__fma_rn(-q, b, a), rb, q);
+}
+__device__ __forceinline__ float div_by(float a, float b, float) { return fdiv(a, b); }
+
 // Sums and products whose rounding the source fixes, whatever kernel they are inlined into:
 // FP32 fuses a b + c into one fma; FP64 rounds the product and the sum separately, as the
 // FP64 build (compiled without contraction) does for every expression.
@@ -244,12 +254,12 @@ __device__ __forceinline__ DF df_sqrt(DF a) {
 __device__ __forceinline__ double psi_eos(const Phys& ph, double rho, double T, double& rad) {
   const double cs2 = 1.0 / 3.0;
   const PhysC<double>& k = ph.d;
-  double s = 1.0 + k.kappa * (1.0 - sqrt(T / k.Tc));
+  double s = 1.0 + k.kappa * (1.0 - sqrt(div_by(T, k.Tc, ph.rTc)));
   double phi = s * s;
   double rep = rho * k.R * T / (1.0 - k.b * rho);
   double att = k.a * phi * rho * rho / (1.0 + 2.0 * k.b * rho - k.b * k.b * rho * rho);
   double p = rep - att;
-  rad = 2.0 * (p - rho * cs2) / (k.G * cs2);
+  rad = div_by(2.0 * (p - rho * cs2), k.G * cs2, ph.rGc);
   return sqrt(rad);
 }
 // The same in double-float arithmetic (inputs and result FP32), over one denominator: with
@@ -319,7 +329,7 @@ __device__ __forceinline__ C dpdT_eos(const Phys& ph, C rho, C T) {
 template <typename C>
 __device__ __forceinline__ C phase_frac(const Phys& ph, C rho) {
   if (!(pc<C>(ph).rho_l > pc<C>(ph).rho_v)) return C(1);
-  C f = fdiv(sub(rho, pc<C>(ph).rho_v), sub(pc<C>(ph).rho_l, pc<C>(ph).rho_v));
+  C f = div_by(sub(rho, pc<C>(ph).rho_v), sub(pc<C>(ph).rho_l, pc<C>(ph).rho_v), C(ph.rdr));
   f = f < C(0) ? C(0) : f;
   return f > C(1) ? C(1) : f;
 }
@@ -476,62 +486,73 @@ __device__ __forceinline__ C psi_node(const Geo& g, const Phys& ph, const S* __r
 // ---------------------------------------------------------------- CM collision (Sec. II.A-B)
 // Raw moments -> central moments k4, k5 (T = N M), post-collision CMs of Eq. (postColl2),
 // m* = N(u)^{-1} k* by forward substitution, f* = M^{-1} m*.  Closed form of the 9x9
-// algebra, term order as in the matrix products.
+// algebra, sums in the order of the matrix products.  FP64: products by powers of two are exact, so
+// they are moved out of the rounded products or into an FMA with the sum, with the same result.
 template <typename C>
 __device__ __forceinline__ void collide(const C f[9], C rho, C Fx, C Fy, C Fmx, C Fmy, C psi, C omega, C sigma,
-                                        C fs[9], C& ux, C& uy) {
-  const C m1 = ((((f[1] - f[2]) + f[5]) - f[6]) + f[7]) - f[8];
-  const C m2 = ((((f[3] - f[4]) + f[5]) - f[6]) - f[7]) + f[8];
-  const C m4 = ((f[1] + f[2]) - f[3]) - f[4];
-  const C m5 = ((f[5] + f[6]) - f[7]) - f[8];
-  ux = fdiv(m1 + C(0.5) * Fx, rho);
-  uy = fdiv(m2 + C(0.5) * Fy, rho);
-  const C u = ux, v = uy;
-  // shift matrix N(u), App. A
-  const C N10 = -u, N20 = -v;
-  const C N30 = u * u + v * v, N31 = C(-2) * u, N32 = C(-2) * v;
-  const C N40 = u * u - v * v, N41 = C(-2) * u, N42 = C(2) * v;
-  const C N50 = u * v, N51 = -v, N52 = -u;
-  const C N60 = -u * u * v, N61 = C(2) * u * v, N62 = u * u, N63 = -v / C(2), N64 = -v / C(2), N65 = C(-2) * u;
-  const C N70 = -u * v * v, N71 = v * v, N72 = C(2) * u * v, N73 = -u / C(2), N74 = u / C(2), N75 = C(-2) * v;
-  const C N80 = u * u * v * v, N81 = C(-2) * u * v * v, N82 = C(-2) * u * u * v, N83 = (u * u + v * v) / C(2),
-          N84 = -(u * u - v * v) / C(2), N85 = C(4) * u * v, N86 = C(-2) * v, N87 = C(-2) * u;
-  const C k4 = ((N40 * rho + N41 * m1) + N42 * m2) + m4;
-  const C k5 = ((N50 * rho + N51 * m1) + N52 * m2) + m5;
+                                        C fs[9], C& ux, C& uy);
+template <>
+__device__ __forceinline__ void collide<double>(const double f[9], double rho, double Fx, double Fy, double Fmx,
+                                                double Fmy, double psi, double omega, double sigma, double fs[9],
+                                                double& ux, double& uy) {
+  const double m1 = ((((f[1] - f[2]) + f[5]) - f[6]) + f[7]) - f[8];
+  const double m2 = ((((f[3] - f[4]) + f[5]) - f[6]) - f[7]) + f[8];
+  const double m4 = ((f[1] + f[2]) - f[3]) - f[4];
+  const double m5 = ((f[5] + f[6]) - f[7]) - f[8];
+  const double ir = 1.0 / rho;
+  ux = div_by(__fma_rn(0.5, Fx, m1), rho, ir);
+  uy = div_by(__fma_rn(0.5, Fy, m2), rho, ir);
+  const double u = ux, v = uy;
+  // entries of the shift matrix N(u), App. A, up to sign and powers of two
+  const double uu = u * u, vv = v * v, uv = u * v, s2 = uu + vv, d2 = uu - vv, uuv = uu * v, uvv = uv * v;
+  const double k4 = __fma_rn(2.0, v * m2, __fma_rn(-2.0, u * m1, d2 * rho)) + m4;
+  const double k5 = ((uv * rho - v * m1) - u * m2) + m5;
   // post-collision central moments
-  const C alpha = sigma != C(0) ? fdiv(sigma, psi * psi) : C(0);
-  const C Fm2 = Fmx * Fmx + Fmy * Fmy;
-  const C ks0 = rho;
-  const C ks1 = C(0.5) * Fx;
-  const C ks2 = C(0.5) * Fy;
-  const C ks3 = fdiv(C(2) * rho, C(3)) + C(0.5) * (C(4) * alpha * Fm2);
-  const C ks4 = (C(1) - omega) * k4;
-  const C ks5 = (C(1) - omega) * k5;
-  const C ks6 = C(0.5) * fdiv(Fy, C(3));
-  const C ks7 = C(0.5) * fdiv(Fx, C(3));
-  const C ks8 = fdiv(rho, C(9)) + C(0.5) * (C(4.0 / 3.0) * alpha * Fm2);
+  const double alpha = sigma != 0.0 ? sigma / (psi * psi) : 0.0;
+  const double Fm2 = Fmx * Fmx + Fmy * Fmy;
+  const double ks3 = 2.0 * (div_by(rho, 3.0, 1.0 / 3.0) + alpha * Fm2);
+  const double ks4 = (1.0 - omega) * k4;
+  const double ks5 = (1.0 - omega) * k5;
+  const double fy3 = div_by(Fy, 3.0, 1.0 / 3.0), fx3 = div_by(Fx, 3.0, 1.0 / 3.0);
+  const double ks8 = __fma_rn(0.5, (4.0 / 3.0) * alpha * Fm2, div_by(rho, 9.0, 1.0 / 9.0));
   // forward substitution N m* = k*
-  const C ms0 = ks0;
-  const C ms1 = ks1 - N10 * ms0;
-  const C ms2 = ks2 - N20 * ms0;
-  const C ms3 = ((ks3 - N30 * ms0) - N31 * ms1) - N32 * ms2;
-  const C ms4 = ((ks4 - N40 * ms0) - N41 * ms1) - N42 * ms2;
-  const C ms5 = ((ks5 - N50 * ms0) - N51 * ms1) - N52 * ms2;
-  const C ms6 = (((((ks6 - N60 * ms0) - N61 * ms1) - N62 * ms2) - N63 * ms3) - N64 * ms4) - N65 * ms5;
-  const C ms7 = (((((ks7 - N70 * ms0) - N71 * ms1) - N72 * ms2) - N73 * ms3) - N74 * ms4) - N75 * ms5;
-  const C ms8 =
-      (((((((ks8 - N80 * ms0) - N81 * ms1) - N82 * ms2) - N83 * ms3) - N84 * ms4) - N85 * ms5) - N86 * ms6) - N87 * ms7;
+  const double ms0 = rho;
+  const double ms1 = __fma_rn(0.5, Fx, u * ms0);
+  const double ms2 = __fma_rn(0.5, Fy, v * ms0);
+  const double p1 = u * ms1, p2 = v * ms2;
+  const double ms3 = __fma_rn(2.0, p2, __fma_rn(2.0, p1, ks3 - s2 * ms0));
+  const double ms4 = __fma_rn(-2.0, p2, __fma_rn(2.0, p1, ks4 - d2 * ms0));
+  const double ms5 = ((ks5 - uv * ms0) + v * ms1) + u * ms2;
+  double t = __fma_rn(0.5, fy3, uuv * ms0);
+  t = __fma_rn(-2.0, uv * ms1, t) - uu * ms2;
+  t = __fma_rn(0.5, v * ms4, __fma_rn(0.5, v * ms3, t));
+  const double ms6 = __fma_rn(2.0, u * ms5, t);
+  t = __fma_rn(0.5, fx3, uvv * ms0);
+  t = __fma_rn(-2.0, uv * ms2, t - vv * ms1);
+  t = __fma_rn(-0.5, u * ms4, __fma_rn(0.5, u * ms3, t));
+  const double ms7 = __fma_rn(2.0, v * ms5, t);
+  t = ks8 - uuv * v * ms0;
+  t = __fma_rn(2.0, uuv * ms2, __fma_rn(2.0, uvv * ms1, t));
+  t = __fma_rn(0.5, d2 * ms4, __fma_rn(-0.5, s2 * ms3, t));
+  t = __fma_rn(2.0, v * ms6, __fma_rn(-4.0, uv * ms5, t));
+  const double ms8 = __fma_rn(2.0, u * ms7, t);
   // f* = M^{-1} m*
-  const C h = C(0.5), q = C(0.25);
+  const double h1 = 0.5 * ms1, h2 = 0.5 * ms2, q5 = 0.25 * ms5;
+  auto axis = [&](double a, double s34, double s6) {  // ((a + ms3 / 4) +/- ms4 / 4) +/- ms_6,7 / 2) - ms8 / 2
+    return __fma_rn(-0.5, ms8, __fma_rn(0.5, s6, __fma_rn(s34, ms4, __fma_rn(0.25, ms3, a))));
+  };
+  auto diag = [&](double a, double s6, double s7) {
+    return __fma_rn(0.25, ms8, __fma_rn(s7, ms7, __fma_rn(s6, ms6, a)));
+  };
   fs[0] = (ms0 - ms3) + ms8;
-  fs[1] = (((h * ms1 + q * ms3) + q * ms4) - h * ms7) - h * ms8;
-  fs[2] = (((-h * ms1 + q * ms3) + q * ms4) + h * ms7) - h * ms8;
-  fs[3] = (((h * ms2 + q * ms3) - q * ms4) - h * ms6) - h * ms8;
-  fs[4] = (((-h * ms2 + q * ms3) - q * ms4) + h * ms6) - h * ms8;
-  fs[5] = ((q * ms5 + q * ms6) + q * ms7) + q * ms8;
-  fs[6] = ((q * ms5 - q * ms6) - q * ms7) + q * ms8;
-  fs[7] = ((-q * ms5 - q * ms6) + q * ms7) + q * ms8;
-  fs[8] = ((-q * ms5 + q * ms6) - q * ms7) + q * ms8;
+  fs[1] = axis(h1, 0.25, -ms7);
+  fs[2] = axis(-h1, 0.25, ms7);
+  fs[3] = axis(h2, -0.25, -ms6);
+  fs[4] = axis(-h2, -0.25, ms6);
+  fs[5] = diag(q5, 0.25, 0.25);
+  fs[6] = diag(q5, -0.25, -0.25);
+  fs[7] = diag(-q5, -0.25, 0.25);
+  fs[8] = diag(-q5, 0.25, -0.25);
 }
 // The same for FP32 with every rounding written out (explicit fma, mul, add), so that the
 // result does not depend on which kernel inlines it.  Forward substitution of N(u) m* = k*
@@ -623,10 +644,10 @@ __device__ __forceinline__ void collide_bgk(const C f[9], C rho, C Fx, C Fy, C o
   const C ks0 = omega * rho;
   const C ks1 = cf * Fx;
   const C ks2 = cf * Fy;
-  const C ks3 = omega * fdiv(C(2) * rho, C(3));
-  const C ks6 = cf * fdiv(Fy, C(3));
-  const C ks7 = cf * fdiv(Fx, C(3));
-  const C ks8 = omega * fdiv(rho, C(9));
+  const C ks3 = omega * div_by(C(2) * rho, C(3), C(1.0 / 3.0));
+  const C ks6 = cf * div_by(Fy, C(3), C(1.0 / 3.0));
+  const C ks7 = cf * div_by(Fx, C(3), C(1.0 / 3.0));
+  const C ks8 = omega * div_by(rho, C(9), C(1.0 / 9.0));
   // forward substitution N m' = k' (k'_4 = k'_5 = 0)
   const C ms0 = ks0;
   const C ms1 = ks1 - N10 * ms0;
@@ -699,7 +720,8 @@ __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const
                                              const uint8_t* __restrict__ mask, const C* __restrict__ side_in,
                                              C* __restrict__ side_out, C* __restrict__ rho_o, C* __restrict__ ux_o,
                                              C* __restrict__ uy_o, int forcing, int* status, int tx, int ty, int x,
-                                             int y, uint8_t m, bool staged, const S* s_f, const C* s_psi) {
+                                             int y, uint8_t m, bool staged, const S* s_f, const C* s_psi,
+                                             C* __restrict__ lam_o) {
   using CS = CollStage<C, S, CTY>;
   constexpr int HX = CS::PW;
   const PhysC<C>& k = pc<C>(ph);
@@ -708,6 +730,7 @@ __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const
     rho_o[id] = k.rho_s;
     ux_o[id] = C(0);
     uy_o[id] = C(0);
+    if (lam_o) lam_o[id] = lam_of(ph, k.rho_s);
     return;
   }
   const bool multiphase = k.G != C(0);
@@ -740,7 +763,7 @@ __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const
     if (k.body_fx != C(0)) Fx = add(Fx, k.body_fx);
     Fy = Fmy;
   }
-  const C omega = fdiv(C(1), add(fdiv(nu_of(ph, rho), cs2), C(0.5)));
+  const C omega = fdiv(C(1), add(div_by(nu_of(ph, rho), cs2, C(1.0 / (1.0 / 3.0))), C(0.5)));
   const C sig = need_psi ? k.sigma : C(0);
   C fs[9], ux, uy;
   if constexpr (OP == kCollBGK) collide_bgk(fo, rho, Fx, Fy, omega, fs, ux, uy);
@@ -750,6 +773,7 @@ __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const
   rho_o[id] = rho;
   ux_o[id] = ux;
   uy_o[id] = uy;
+  if (lam_o) lam_o[id] = lam_of(ph, rho);
   if (!(rho > C(0)) || !(ux == ux) || !(uy == uy)) atomicOr(status, 1);
 }
 
@@ -772,7 +796,7 @@ __device__ __forceinline__ void collide_tile(const Geo& g, const Phys& ph, const
                                              C* __restrict__ side_out, C* __restrict__ rho_o, C* __restrict__ ux_o,
                                              C* __restrict__ uy_o, int forcing, int* status, int bx, int by,
                                              const CUtensorMap* tm_f = nullptr, const CUtensorMap* tm_psi = nullptr,
-                                             bool starve = false, bool early_f = false) {
+                                             bool starve = false, bool early_f = false, C* lam_o = nullptr) {
   using CS = CollStage<C, S, CTY>;
   constexpr int HX = CS::PW, HY = CS::PH;
   __shared__ __align__(128) S s_f[9 * CS::FH * CS::FW];
@@ -818,7 +842,7 @@ __device__ __forceinline__ void collide_tile(const Geo& g, const Phys& ph, const
   }
   if (!inside) return;
   collide_node<C, S, CTY, OP>(g, ph, f, fn, psi, mask, side_in, side_out, rho_o, ux_o, uy_o, forcing, status, tx, ty,
-                              x, y, m, staged, s_f, s_psi);
+                              x, y, m, staged, s_f, s_psi, lam_o);
 }
 
 template <typename C, typename S, int OP = kCollCM>
@@ -829,11 +853,12 @@ __global__ void __launch_bounds__(kCollTX* kCollTY, sizeof(C) == 4 ? 7 : 1)
     k_collide(Geo g, Phys ph, const S* __restrict__ f, S* __restrict__ fn, const C* __restrict__ psi,
               const uint8_t* __restrict__ mask, const C* __restrict__ side_in, C* __restrict__ side_out,
               C* __restrict__ rho_o, C* __restrict__ ux_o, C* __restrict__ uy_o, int forcing, int* status,
-              const __grid_constant__ CUtensorMap tm_f, const __grid_constant__ CUtensorMap tm_psi, int flags) {
+              const __grid_constant__ CUtensorMap tm_f, const __grid_constant__ CUtensorMap tm_psi, int flags,
+              C* __restrict__ lam_o) {
   const bool staged = flags & kLaunchStaged;
   collide_tile<C, S, kCollTY, OP>(g, ph, f, fn, psi, mask, side_in, side_out, rho_o, ux_o, uy_o, forcing, status,
                                   blockIdx.x, blockIdx.y, staged ? &tm_f : nullptr, staged ? &tm_psi : nullptr,
-                                  (flags & kLaunchStarve) != 0, (flags & kLaunchEarlyF) != 0);
+                                  (flags & kLaunchStarve) != 0, (flags & kLaunchEarlyF) != 0, lam_o);
 }
 
 // ---------------------------------------------------------------- k_energy
@@ -1400,6 +1425,37 @@ __global__ void __launch_bounds__(EnergyTile<C>::NT, sizeof(C) == 4 ? (sizeof(S)
                                                    (flags & kLaunchStarve) != 0);
 }
 
+}  // namespace kern
+}  // namespace lbm
+#include "lbm_energy_f64.cuh"
+namespace lbm {
+namespace kern {
+
+// Planes of the FP64 energy pass in a context's work planes (T1 first).
+__device__ __forceinline__ Frozen64 frozen64(double* en64, const Geo& g) {
+  const size_t n = g.plane;
+  return {en64 + n, en64 + 2 * n, en64 + 3 * n, en64 + 4 * n, en64 + 5 * n, en64 + 6 * n};
+}
+static __global__ void __launch_bounds__(128)
+    k_energy1_f64(Geo g, Phys ph, const double* __restrict__ Tin, double* __restrict__ T1, double* en64,
+                  const double* __restrict__ lam, const double* __restrict__ rho, const double* __restrict__ ux,
+                  const double* __restrict__ uy, const uint8_t* __restrict__ mask, double* partial, unsigned* counter,
+                  double* hf, int nb, int do_hf, int n_wall_tiles, int* status, const __grid_constant__ EnergyMaps maps,
+                  int flags) {
+  energy1_tile(g, ph, Tin, T1, lam, frozen64(en64, g), rho, ux, uy, mask, partial, counter, hf, nb, do_hf, n_wall_tiles,
+               blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y, status,
+               (flags & kLaunchStaged) ? &maps : nullptr, (flags & kLaunchStarve) != 0);
+}
+static __global__ void __launch_bounds__(128)
+    k_energy2_f64(Geo g, Phys ph, const double* __restrict__ Tin, double* __restrict__ Tout,
+                  const double* __restrict__ T1, double* en64, const double* __restrict__ lam,
+                  const double* __restrict__ rho, const double* __restrict__ ux, const double* __restrict__ uy,
+                  const uint8_t* __restrict__ mask, const double* __restrict__ fnew,
+                  const double* __restrict__ side_new, double* __restrict__ psi_out, int* status) {
+  energy2_tile(g, ph, Tin, Tout, T1, lam, frozen64(en64, g), rho, ux, uy, mask, blockIdx.x, blockIdx.y, fnew, side_new,
+               psi_out, status);
+}
+
 // ---------------------------------------------------------------- batched passes
 // Every block of a batched pass finds its domain through the block -> domain map and its
 // tile from its index within that domain; the tile bodies are the single-domain ones.
@@ -1434,7 +1490,53 @@ __global__ void __launch_bounds__(kCollTX* CTY, (sizeof(C) == 4 && CTY == 8) ? 7
                           static_cast<C*>(D.d.side[cur ^ 1]), static_cast<C*>(D.d.rho), static_cast<C*>(D.d.ux),
                           static_cast<C*>(D.d.uy), step >= D.warmup, D.d.status, local % D.coll_ntx,
                           local / D.coll_ntx, D.tma ? &maps.f[k - dom0] : nullptr,
-                          D.tma ? &maps.psi[k - dom0] : nullptr);
+                          D.tma ? &maps.psi[k - dom0] : nullptr, false, false,
+                          sizeof(C) == 8 ? static_cast<C*>(D.d.lam) : nullptr);
+}
+// FP64 energy pass of a batch: the two stages of the domains that take an energy step; the others
+// carry T over in the second.
+static __global__ void __launch_bounds__(128)
+    kb_energy1_f64(const BatchDomain* __restrict__ doms, const int* __restrict__ map, int tcur, long long step, int block0,
+                   int dom0, const __grid_constant__ EnLaunchMaps maps) {
+  const int blk = block0 + blockIdx.x, k = map[blk];
+  const BatchDomain& D = doms[k];
+  const int local = blk - D.en_first;
+  if (!D.energy || step < D.warmup) return;
+  energy1_tile(D.g, D.ph, static_cast<const double*>(D.d.T[tcur]), static_cast<double*>(D.d.en64),
+               static_cast<const double*>(D.d.lam), frozen64(static_cast<double*>(D.d.en64), D.g),
+               static_cast<const double*>(D.d.rho), static_cast<const double*>(D.d.ux),
+               static_cast<const double*>(D.d.uy), D.d.mask, D.d.partial, D.d.counter, D.d.hf, D.d.nb, D.d.nb > 0,
+               D.d.wall_tiles[0], local % D.en_ntx, local / D.en_ntx, local, D.en_nblocks, D.d.status,
+               D.tma ? &maps.e[k - dom0] : nullptr, false);
+}
+static __global__ void __launch_bounds__(128)
+    kb_energy2_f64(const BatchDomain* __restrict__ doms, const int* __restrict__ map, int cur, int tcur, long long step) {
+  const int k = map[blockIdx.x];
+  const BatchDomain& D = doms[k];
+  const int local = blockIdx.x - D.en_first, bx = local % D.en_ntx, by = local / D.en_ntx;
+  const double* Tin = static_cast<const double*>(D.d.T[tcur]);
+  double* Tout = static_cast<double*>(D.d.T[tcur ^ 1]);
+  const double* fnew = static_cast<const double*>(D.d.f[cur ^ 1]);
+  const double* side_new = static_cast<const double*>(D.d.side[cur ^ 1]);
+  double* psi_next = D.ph.d.G != 0.0 ? psi_buf<double>(D, cur ^ 1) : nullptr;
+  if (!D.energy || step < D.warmup) {
+    // no energy update for this domain this step: carry T over so all domains flip together,
+    // and make psi of the next state from the new populations and the unchanged T
+    for (int p = threadIdx.x; p < kEnergyTX * 8; p += 128) {
+      const int x = bx * kEnergyTX + p % kEnergyTX, y = by * 8 + p / kEnergyTX;
+      if (x < D.g.nx && y < D.g.ny) {
+        Tout[y * D.g.pitch + x] = Tin[y * D.g.pitch + x];
+        if (psi_next)
+          psi_next[y * D.g.pitch + x] =
+              psi_node<double, double, kPsiF64>(D.g, D.ph, fnew, Tin, D.d.mask, side_new, x, y, D.d.status);
+      }
+    }
+    return;
+  }
+  energy2_tile(D.g, D.ph, Tin, Tout, static_cast<const double*>(D.d.en64), static_cast<const double*>(D.d.lam),
+               frozen64(static_cast<double*>(D.d.en64), D.g), static_cast<const double*>(D.d.rho),
+               static_cast<const double*>(D.d.ux), static_cast<const double*>(D.d.uy), D.d.mask, bx, by, fnew, side_new,
+               psi_next, D.d.status);
 }
 template <typename C, int ETY, int PSI>
 // FP32: a register budget for 1280 threads per SM, as the single-domain energy pass
@@ -1498,7 +1600,12 @@ int batch_step_impl(const BatchDomain* doms, const int* map_psi, int nb_psi, con
     EnLaunchMaps m;
     for (int k = d0; k < d1; ++k) m.e[k - d0] = hmaps[k].em[tcur];
     const int b0 = hdoms[d0].en_first, b1 = d1 < ndom ? hdoms[d1].en_first : nb_en;
-    kb_energy<C, ETY, PSI><<<b1 - b0, EnergyTile<C, ETY>::NT, 0, s>>>(doms, map_en, cur, tcur, step, b0, d0, m);
+    if constexpr (sizeof(C) == 8) kb_energy1_f64<<<b1 - b0, 128, 0, s>>>(doms, map_en, tcur, step, b0, d0, m);
+    else kb_energy<C, ETY, PSI><<<b1 - b0, EnergyTile<C, ETY>::NT, 0, s>>>(doms, map_en, cur, tcur, step, b0, d0, m);
+    ++n;
+  }
+  if constexpr (sizeof(C) == 8) {
+    kb_energy2_f64<<<nb_en, 128, 0, s>>>(doms, map_en, cur, tcur, step);
     ++n;
   }
   return cudaPeekAtLastError() == cudaSuccess ? n : -1;
@@ -1510,15 +1617,16 @@ template <typename C, typename S>
 bool batch_maps_impl(BatchDomain& D, DomainMaps& m, int cty, int ety) {
   const Geo& g = D.g;
   const int XA = 16 / (int)sizeof(S), PA = 16 / (int)sizeof(C) < 2 ? 2 : 16 / (int)sizeof(C);
+  const int EH = sizeof(C) == 8 ? 4 : 8;  // both halos of the energy tile
   bool ok = D.d.tma != 0;
   for (int p = 0; p < 2 && ok; ++p) {
     ok = tma::encode<S>(&m.f[p], D.d.f[p], g.nx, g.ny, g.pitch, g.plane, 9, kCollTX + 2 * XA, cty + 2) &&
          tma::encode<C>(&m.psi[p], p ? D.d.psi_next : D.d.psi, g.nx, g.ny, g.pitch, g.plane, 1,
                         kCollTX + 2 * PA, cty + 4) &&
-         tma::encode<C>(&m.em[p].T, D.d.T[p], g.nx, g.ny, g.pitch, g.plane, 1, kEnergyTX + 8, ety + 8) &&
+         tma::encode<C>(&m.em[p].T, D.d.T[p], g.nx, g.ny, g.pitch, g.plane, 1, kEnergyTX + EH, ety + EH) &&
          static_cast<const C*>(D.d.ux) == static_cast<const C*>(D.d.rho) + g.plane &&
          static_cast<const C*>(D.d.uy) == static_cast<const C*>(D.d.rho) + 2 * (size_t)g.plane &&
-         tma::encode<C>(&m.em[p].ruv, D.d.rho, g.nx, g.ny, g.pitch, g.plane, 3, kEnergyTX + 8, ety + 8);
+         tma::encode<C>(&m.em[p].ruv, D.d.rho, g.nx, g.ny, g.pitch, g.plane, 3, kEnergyTX + EH, ety + EH);
   }
   D.tma = ok ? 1 : 0;
   return ok;
@@ -1723,12 +1831,13 @@ int step_impl(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int
   const int cflags = staged ? (kLaunchStaged | ((d.starve & kStarveCollide) ? kLaunchStarve : 0) |
                                ((d.pdl && d.f_ready) ? kLaunchEarlyF : 0))
                             : 0;
+  C* const lam = sizeof(C) == 8 && energy && forcing ? static_cast<C*>(d.lam) : nullptr;
   if (d.collision == kCollBGK)
     launch_dep(d.pdl, grd, blk, 0, s, k_collide<C, S, kCollBGK>, g, ph, f, fn, psi, d.mask, side_in, side_out, rho, ux,
-               uy, forcing, d.status, tm_f, tm_psi, cflags);
+               uy, forcing, d.status, tm_f, tm_psi, cflags, lam);
   else
     launch_dep(d.pdl, grd, blk, 0, s, k_collide<C, S, kCollCM>, g, ph, f, fn, psi, d.mask, side_in, side_out, rho, ux, uy,
-               forcing, d.status, tm_f, tm_psi, cflags);
+               forcing, d.status, tm_f, tm_psi, cflags, lam);
   post(kKCollide);
   *t_flipped = 0;
   if (energy && forcing) {
@@ -1737,16 +1846,29 @@ int step_impl(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int
     pre(kKEnergy);
     using ET = EnergyTile<C>;
     const dim3 blk(ET::NT), grd((g.nx + ET::TX - 1) / ET::TX, (g.ny + ET::TY - 1) / ET::TY);
-    constexpr int AX = ET::TX + 8, AY = ET::TY + 8;
+    constexpr int EH = sizeof(C) == 8 ? 4 : 8;  // both halos
+    constexpr int AX = ET::TX + EH, AY = ET::TY + EH;
     EnergyMaps em;
     const bool ruv = ux == rho + g.plane && uy == rho + 2 * (size_t)g.plane;  // consecutive planes
     const bool e_staged = d.tma && ruv && tma::encode<C>(&em.T, T, g.nx, g.ny, g.pitch, g.plane, 1, AX, AY) &&
                           tma::encode<C>(&em.ruv, rho, g.nx, g.ny, g.pitch, g.plane, 3, AX, AY);
-    launch_dep(d.pdl, grd, blk, 0, s, k_energy<C, S, PSI>, g, ph, T, Tn, rho, ux, uy, d.mask, d.partial, d.counter,
-               d.hf, d.nb, do_hf, d.wall_tiles[ET::TY == 16 ? 1 : 0], fuse ? static_cast<const S*>(fn) : nullptr,
-               static_cast<const C*>(side_out), fuse ? static_cast<C*>(d.psi_next) : nullptr, d.status,
-               static_cast<C*>(d.t1_out), em,
-               e_staged ? (kLaunchStaged | ((d.starve & kStarveEnergy) ? kLaunchStarve : 0)) : 0);
+    const int eflags = e_staged ? (kLaunchStaged | ((d.starve & kStarveEnergy) ? kLaunchStarve : 0)) : 0;
+    if constexpr (sizeof(C) == 8) {
+      double* en64 = static_cast<double*>(d.en64);
+      double* T1 = d.t1_out ? static_cast<double*>(d.t1_out) : en64;
+      launch_dep(d.pdl, grd, blk, 0, s, k_energy1_f64, g, ph, T, T1, en64, lam, rho, ux, uy, d.mask, d.partial, d.counter,
+                 d.hf, d.nb, do_hf, d.wall_tiles[0], d.status, em, eflags);
+      launch_dep(d.pdl, grd, blk, 0, s, k_energy2_f64, g, ph, T, Tn, T1, en64, lam, rho, ux, uy, d.mask,
+                 fuse ? static_cast<const double*>(fn) : nullptr, side_out,
+                 fuse ? static_cast<double*>(d.psi_next) : nullptr, d.status);
+      ++n;
+    } else {
+      launch_dep(d.pdl, grd, blk, 0, s, k_energy<C, S, PSI>, g, ph, T, Tn, rho, ux, uy, d.mask, d.partial, d.counter,
+                 d.hf, d.nb, do_hf, d.wall_tiles[ET::TY == 16 ? 1 : 0], fuse ? static_cast<const S*>(fn) : nullptr,
+                 static_cast<const C*>(side_out), fuse ? static_cast<C*>(d.psi_next) : nullptr, d.status,
+                 static_cast<C*>(d.t1_out), em,
+                 eflags);
+    }
     post(kKEnergy);
     *t_flipped = 1;
     if (chain) chain->made = fuse ? 1 : 0;
