@@ -74,12 +74,17 @@ POP = {"f32": 4, "f64": 8, "f16s": 2}[next((a.split("=", 1)[1] for a in sys.argv
                                            sys.argv[sys.argv.index("--storage") + 1] if "--storage" in sys.argv else "f32")]
 ALG_BYTES = {
     "k_rho_psi": 9 * POP + 4 + 4,           # f, T in; psi out
-    "k_collide": 9 * POP + 4 + 9 * POP + 12,  # f, psi in; f*, rho, ux, uy out (no psi when single phase)
-    # T, rho, ux, uy in; T out; and psi of the next step: the new populations in, psi out
-    "k_energy": 4 * 4 + 4 + 9 * POP + 4,
+    # FP32 populations: f, T in; f*, rho, ux, uy, psi out (psi is evaluated there: no psi nor T when single
+    # phase); others: f, psi in; f*, rho, ux, uy out
+    "k_collide": 9 * POP + 4 + 9 * POP + 12 + (4 if POP == 4 else 0),
+    # T, rho, ux, uy in; T out; and, where the collision does not make psi, psi of the next step: the new
+    # populations in, psi out
+    "k_energy": 4 * 4 + 4 + (0 if POP == 4 else 9 * POP + 4),
 }
 STEP_ALG_BYTES = 9 * POP * 2 + 4 * 2      # the whole step: populations and T in and out
-KERNEL_SRCS = [os.path.join(ROOT, "paper_1912_02018_gb300", "csrc", n) for n in ("lbm_kernels.cuh", "lbm_tma.cuh")]
+KERNEL_SRCS = [os.path.join(ROOT, "paper_1912_02018_gb300", "csrc", n) for n in (
+    "lbm_kernels.cuh", "lbm_tma.cuh", "lbm_step_f32.cuh", "lbm_flow_f32.cuh", "lbm_energy_f32.cuh", "lbm_energy_f64.cuh",
+    "lbm_step_f16s.cuh")]
 
 
 def kernel_hash() -> str:
@@ -499,7 +504,7 @@ def run_ours(args):
     ours = {k: v for k, v in prof.items() if v[0] > 0}
     dom = max(ours, key=lambda k: ours[k][1])
     per_launch_ms = ours[dom][1] / ours[dom][0]
-    alg_lup = ALG_BYTES.get(dom, 0) - (4 if (dom == "k_collide" and case.G == 0) else 0)
+    alg_lup = ALG_BYTES.get(dom, 0) - ((8 if POP == 4 else 4) if (dom == "k_collide" and case.G == 0) else 0)
     alg = alg_lup * nodes
     achieved = alg / (per_launch_ms / 1e3) / 1e9
     traffic = ncu_traffic(dom, args.workload)

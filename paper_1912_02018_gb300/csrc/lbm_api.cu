@@ -395,6 +395,21 @@ lbm_status lbm_create(const lbm_domain* domain, const lbm_cylinder* cyl, const l
   phys.dpdT_c1 = (float)(eos.kappa * (1.0 + eos.kappa));
   phys.dpdT_c2 = (float)(eos.kappa * eos.kappa / eos.Tc);
   {
+    lbm::StepConst& en = phys.sc;
+    const bool two = rho_l > rho_v;  // else the phase fraction is 1 everywhere
+    en.T_sat = (float)T_sat;
+    en.T_wall = (float)T_wall, en.th_wall = (float)(T_wall - T_sat), en.dT_sat = (float)(T_sat - en.T_sat);
+    en.ph1 = two ? (float)(1.0 / (rho_l - rho_v)) : 0.0f;
+    en.ph0 = two ? (float)(-rho_v / (rho_l - rho_v)) : 1.0f;
+    en.da = (float)(ph.alpha_l - ph.alpha_v), en.av = (float)ph.alpha_v;
+    en.rep = (float)(P.R / P.c_v), en.att = (float)(P.a / P.c_v);
+    en.b = (float)P.b, en.bb = (float)(P.b * P.b), en.b2 = (float)(2.0 * P.b);
+    en.c1 = (float)(eos.kappa * (1.0 + eos.kappa) / std::sqrt(eos.Tc));
+    en.c2 = (float)(eos.kappa * eos.kappa / eos.Tc);
+    en.gm = (float)(-P.G / 3.0), en.sg = (float)(P.sigma * P.G * P.G / 9.0);
+    en.nv3 = (float)(3.0 * ph.nu_v), en.dn3 = (float)(3.0 * (ph.nu_l - ph.nu_v));
+  }
+  {
     static const double W[9] = {4.0 / 9.0, 1.0 / 9.0, 1.0 / 9.0, 1.0 / 9.0, 1.0 / 9.0,
                                 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0};
     for (int i = 0; i < 9; ++i) phys.pop_shift[i] = (float)(W[i] * rho_l);
@@ -520,15 +535,24 @@ lbm_status lbm_create(const lbm_domain* domain, const lbm_cylinder* cyl, const l
       if (near2) mask[id] |= lbm::kNear2;
     }
 
-  // energy tiles (32 x 8 and 32 x 16) that hold a near-wall node: they alone sum heat flux
-  int wall_tiles[2] = {0, 0};
-  for (int h = 0; h < 2; ++h) {
-    const int TY = h == 0 ? 8 : 16;
+  g.hf_g0 = g.hf_g1 = 0;
+  for (int y = 0; y < g.ny; ++y)
+    for (int x = 0; x < g.nx; ++x)
+      if (mask[(long long)y * g.pitch + x] & lbm::kNearWall) {
+        if (!g.hf_g1) g.hf_g0 = y / 4;
+        g.hf_g1 = y / 4 + 1;
+        break;
+      }
+  // energy tiles (8, 16 and 4 rows high) that hold a near-wall node: they alone sum heat flux
+  int wall_tiles[3] = {0, 0, 0};
+  const int TX = c->f64 || P.storage == LBM_STORE_F16S ? lbm::kEnergyTX64 : lbm::kEnergyTX32;
+  for (int h = 0; h < 3; ++h) {
+    const int TY = h == 0 ? 8 : (h == 1 ? lbm::kEnergyTY : lbm::kEnergyTYSmall);
     for (int ty = 0; ty * TY < g.ny; ++ty)
-      for (int tx = 0; tx * 32 < g.nx; ++tx) {
+      for (int tx = 0; tx * TX < g.nx; ++tx) {
         bool any = false;
         for (int y = ty * TY; y < std::min(g.ny, ty * TY + TY) && !any; ++y)
-          for (int x = tx * 32; x < std::min(g.nx, tx * 32 + 32) && !any; ++x)
+          for (int x = tx * TX; x < std::min(g.nx, tx * TX + TX) && !any; ++x)
             any = (mask[(long long)y * g.pitch + x] & lbm::kNearWall) != 0;
         wall_tiles[h] += any ? 1 : 0;
       }
@@ -559,6 +583,7 @@ lbm_status lbm_create(const lbm_domain* domain, const lbm_cylinder* cyl, const l
   d.counter = static_cast<unsigned*>(dalloc(c, sizeof(unsigned)));
   d.wall_tiles[0] = wall_tiles[0];
   d.wall_tiles[1] = wall_tiles[1];
+  d.wall_tiles[2] = wall_tiles[2];
   uint8_t* dmask = static_cast<uint8_t*>(dalloc(c, N));
   d.mask = dmask;
   d.nb = (int)bnode.size();
@@ -1024,11 +1049,12 @@ static lbm_status batch_layout(lbm_batch* b) {
     D.psi_ntx = ntx;
     mp.insert(mp.end(), (size_t)ntx * ((g.ny + 7) / 8), (int)k);
     D.coll_first = (int)mc.size();
-    D.coll_ntx = ntx;
-    mc.insert(mc.end(), (size_t)ntx * ((g.ny + cty - 1) / cty), (int)k);
+    D.coll_ntx = b->f64 ? ntx : (g.nx + lbm::kFlowTX - 1) / lbm::kFlowTX;
+    mc.insert(mc.end(), (size_t)D.coll_ntx * ((g.ny + cty - 1) / cty), (int)k);
     D.en_first = (int)me.size();
-    D.en_ntx = ntx;
-    D.en_nblocks = ntx * ((g.ny + ety - 1) / ety);
+    const int etx = b->f64 ? lbm::kEnergyTX64 : lbm::kEnergyTX32;
+    D.en_ntx = (g.nx + etx - 1) / etx;
+    D.en_nblocks = D.en_ntx * ((g.ny + ety - 1) / ety);
     me.insert(me.end(), (size_t)D.en_nblocks, (int)k);
     // TMA maps for this variant's tiles (plain loads for the domain when one cannot be made)
     if (b->f64) lbm::batch_maps_f64(D, b->hmaps[k], cty, ety);

@@ -86,7 +86,7 @@ __device__ __forceinline__ void energy1_tile(const Geo& g, const Phys& ph, const
                                              const uint8_t* __restrict__ mask, double* partial, unsigned* counter,
                                              double* hf, int nb, int do_hf, int n_wall_tiles, int bx, int by, int bid,
                                              int nblocks, int* status, const EnergyMaps* maps, bool starve) {
-  constexpr int TX = kEnergyTX, TY = 8, H = 2, AX = TX + 2 * H, AY = TY + 2 * H, NT = TX * TY / 2;
+  constexpr int TX = kEnergyTX64, TY = 8, H = 2, AX = TX + 2 * H, AY = TY + 2 * H, NT = TX * TY / 2;
   __shared__ __align__(128) double sT[AY * AX];
   __shared__ __align__(128) double sRUV[3 * AY * AX];  // rho, u_x, u_y: the planes of one TMA box
   __shared__ __align__(16) double sL[AY * AX];
@@ -202,7 +202,7 @@ __device__ __forceinline__ void energy2_tile(const Geo& g, const Phys& ph, const
                                              int* status) {
   pdl::wait();  // T1 and the frozen parts are the previous kernel's output
   pdl::trigger();
-  const int x0 = bx * kEnergyTX + (threadIdx.x % (kEnergyTX / 2)) * 2, y = by * 8 + threadIdx.x / (kEnergyTX / 2);
+  const int x0 = bx * kEnergyTX64 + (threadIdx.x % (kEnergyTX64 / 2)) * 2, y = by * 8 + threadIdx.x / (kEnergyTX64 / 2);
   if (x0 >= g.nx || y >= g.ny) return;
   const int id = y * g.pitch + x0;
   double w[5][6], tnew[2];

@@ -3,7 +3,7 @@
 // (IEEE FP64 or plain FP32 on request) and the wall heat flux is accumulated in FP64.
 #include "lbm.h"
 #include "lbm_adjoint.cuh"
-#include "lbm_kernels.cuh"
+#include "lbm_step_f32.cuh"
 
 namespace lbm {
 
@@ -11,10 +11,18 @@ namespace {
 template <typename S>
 int step_s(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int forcing, int energy, int psi_mode,
            cudaStream_t s, const LaunchHook* hook, int* t_flipped, PsiChain* chain) {
-  switch (psi_mode) {
-    case kPsiF64: return step_impl<float, S, kPsiF64>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
-    case kPsiF32: return step_impl<float, S, kPsiF32>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
-    default: return step_impl<float, S, kPsiDF>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
+  if constexpr (sizeof(S) == 2) {
+    switch (psi_mode) {
+      case kPsiF64: return step_impl<float, S, kPsiF64>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
+      case kPsiF32: return step_impl<float, S, kPsiF32>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
+      default: return step_impl<float, S, kPsiDF>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
+    }
+  } else {
+    switch (psi_mode) {
+      case kPsiF64: return step_impl_f32<S, kPsiF64>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
+      case kPsiF32: return step_impl_f32<S, kPsiF32>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
+      default: return step_impl_f32<S, kPsiDF>(g, ph, d, cur, tcur, forcing, energy, s, hook, t_flipped, chain);
+    }
   }
 }
 }  // namespace
@@ -53,17 +61,17 @@ int init_f32(const Geo& g, const Phys& ph, const Dev& d, const double* rho0, con
 }
 
 bool batch_maps_f32(BatchDomain& D, DomainMaps& m, int cty, int ety) {
-  return kern::batch_maps_impl<float, float>(D, m, cty, ety);
+  return kern::batch_maps_impl_f32(D, m, cty, ety);
 }
 
-int batch_step_f32(int variant, const BatchDomain* doms, const int* mp, int np, const int* mc, int nc,
-                   const int* me, int ne, int cur, int tcur, long long step, int need_psi,
-                   const BatchDomain* hd, const DomainMaps* hm, int nd, cudaStream_t s) {
+int batch_step_f32(int variant, const BatchDomain* doms, const int*, int, const int* mc, int nc, const int* me, int ne,
+                   int cur, int tcur, long long step, int, const BatchDomain* hd, const DomainMaps* hm, int nd,
+                   cudaStream_t s) {
   switch (variant) {
-    case 1: return kern::batch_step_impl<float, float, kPsiDF, 16, 16>(doms, mp, np, mc, nc, me, ne, cur, tcur, step, need_psi, hd, hm, nd, s);
-    case 2: return kern::batch_step_impl<float, float, kPsiDF, 8, 8>(doms, mp, np, mc, nc, me, ne, cur, tcur, step, need_psi, hd, hm, nd, s);
-    case 3: return kern::batch_step_impl<float, float, kPsiDF, 16, 8>(doms, mp, np, mc, nc, me, ne, cur, tcur, step, need_psi, hd, hm, nd, s);
-    default: return kern::batch_step_impl<float, float, kPsiDF, 8, 16>(doms, mp, np, mc, nc, me, ne, cur, tcur, step, need_psi, hd, hm, nd, s);
+    case 1: return kern::batch_step_impl_f32<8, 16>(doms, mc, nc, me, ne, cur, tcur, step, hd, hm, nd, s);
+    case 2: return kern::batch_step_impl_f32<kFlowTY, 8>(doms, mc, nc, me, ne, cur, tcur, step, hd, hm, nd, s);
+    case 3: return kern::batch_step_impl_f32<8, 8>(doms, mc, nc, me, ne, cur, tcur, step, hd, hm, nd, s);
+    default: return kern::batch_step_impl_f32<kFlowTY, 16>(doms, mc, nc, me, ne, cur, tcur, step, hd, hm, nd, s);
   }
 }
 

@@ -18,6 +18,7 @@ constexpr uint8_t kNear2 = 4;     // fluid node with a solid node at most 2 node
 struct Geo {
   int nx, ny, pitch, periodic_x;
   int plane;        // elements per population plane = ny * pitch (9 * plane < 2^31)
+  int hf_g0, hf_g1; // the 4-row groups [hf_g0, hf_g1) of the lattice that hold near-wall nodes
   double xc, yc, r; // cylinder centre and radius (r <= 0: none)
   // link fractions of the near-wall nodes, tabulated on the host: wall_idx[y * pitch + x] is
   // the node's row (-1 away from the wall); wall_q[row * 8 + i - 1] (compute type) is the
@@ -45,6 +46,15 @@ struct PhysC {
   C body_fx;  // uniform body force along +x (0: none)
 };
 
+// Constants of the FP32 passes: phase fraction = clamp(rho ph1 + ph0).  Energy: T_sat, T_wall as
+// stored, T_wall - T_sat rounded from FP64, and what the stored T_sat lacks of it; alpha = av +
+// da times the fraction; R / c_v, a / c_v, b, b^2, 2 b of the EOS; kappa (1 + kappa) / sqrt(Tc),
+// kappa^2 / Tc.  Collision: -G / 3, sigma (G / 3)^2, and 3 nu = nv3 + dn3 times the fraction.
+struct StepConst {
+  float T_sat, T_wall, th_wall, dT_sat, ph1, ph0, da, av, rep, att, b, bb, b2, c1, c2;
+  float gm, sg, nv3, dn3;
+};
+
 // Physical constants, derived on the host in double and rounded once to float there, so
 // that no kernel converts a double to a float (on GB300 that conversion runs on the FP64
 // pipe).  The double-float copies serve the FP32 build's psi: a, b, R, kappa, 1/Tc,
@@ -55,8 +65,9 @@ struct Phys {
   F2 a2, b2, R2, kappa2, invTc2, cs22, k2;
   F2 kR2, ka2, k32;  // k R, k a, k / 3 with k = 2 / (G cs^2): the double-float psi's folded constants
   F2 K12;            // 1 + kappa (the same)
-  float dpdT_c1, dpdT_c2;  // kappa (1 + kappa) and kappa^2 / Tc: (dp/dT)_rho of the FP32 energy pass
+  float dpdT_c1, dpdT_c2;  // kappa (1 + kappa) and kappa^2 / Tc: (dp/dT)_rho of the FP16-storage energy pass
   double rTc, rdr, rGc;  // 1 / T_c, 1 / (rho_l - rho_v), 1 / (G cs^2): reciprocals of the FP64 divisors
+  StepConst sc;
   float pop_shift[9];  // shifted FP16 storage keeps f_i - w_i rho_l; these are w_i rho_l
 };
 
@@ -102,7 +113,7 @@ struct Dev {
   int collision;     // LBM_COLL_CM or LBM_COLL_BGK
   double* hf;        // heat-flux accumulators: last, sum, sum of squares, count
   double* partial;   // one heat-flux partial sum per energy-kernel block (zero between launches)
-  int wall_tiles[2]; // energy tiles (32 wide, 8 or 16 high) that hold a near-wall node
+  int wall_tiles[3]; // energy tiles (8, 16 or 4 high, as wide as the precision's) that hold a near-wall node
   unsigned* counter; // blocks of the current energy launch that have finished (wraps to 0)
   int* status;       // latched fault bits
   double* stage;     // nx*ny doubles for exports/imports
@@ -150,10 +161,12 @@ struct EnLaunchMaps {
 bool batch_maps_f32(BatchDomain& D, DomainMaps& m, int cty, int ety);
 bool batch_maps_f64(BatchDomain& D, DomainMaps& m, int cty, int ety);
 
+// FP32 collision tiles with psi: 60 x 12 nodes (48 KB of shared memory).
+constexpr int kFlowTX = 60, kFlowTY = 12;
 // Tile-height variants of the batched step the autotuner chooses from: (CTY, ETY).
 constexpr int kBatchVariants = 4;
 inline void batch_variant(int v, bool f64, int& cty, int& ety) {
-  cty = (v & 1) ? 16 : 8;
+  cty = f64 ? ((v & 1) ? 16 : 8) : ((v & 1) ? 8 : kFlowTY);
   ety = f64 ? 8 : ((v & 2) ? 8 : 16);
 }
 
@@ -171,10 +184,16 @@ int batch_step_f64(int variant, const BatchDomain* doms, const int* map_psi, int
 // Kernel identifiers for per-launch timing.
 enum KernelId { kKRhoPsi = 0, kKCollide, kKEnergy, kKExport, kKImport, kNumKernels };
 
-// Tile shapes (threads per block = tile nodes).
-constexpr int kEnergyTX = 32, kEnergyTY = 16;
-inline int energy_blocks(int nx, int ny) {  // upper bound over both precisions (FP64 tiles are 32x8)
-  return ((nx + kEnergyTX - 1) / kEnergyTX) * ((ny + 7) / 8);
+// Energy tiles: 32 x 8 nodes in FP64, 32 x 16 with FP16 storage, else 60 x 16 (4, 8) in FP32.
+constexpr int kEnergyTX64 = 32, kEnergyTX32 = 60, kEnergyTY = 16, kEnergyTYSmall = 4;
+// Small lattices: fewer 60 x 16 energy tiles than SMs; the energy pass then takes 4-row tiles (four
+// times the blocks, each less than half as long: the pass is one wave either way).
+inline bool small_lattice(int nx, int ny) { return (long long)((nx + 59) / 60) * ((ny + 15) / 16) < 152; }
+// Lattices whose first FP32 step evaluates psi in the collision's tiles too (no psi pass at all); on
+// smaller ones that pass is 3 us of one step.
+inline bool flow_psi_in_tile(int nx, int ny) { return (long long)nx * ny >= 12000; }
+inline int energy_blocks(int nx, int ny) {  // upper bound over both precisions
+  return ((nx + kEnergyTX64 - 1) / kEnergyTX64) * ((ny + 3) / 4);
 }
 extern const char* const kKernelNames[kNumKernels];
 
@@ -185,9 +204,9 @@ struct LaunchHook {
   void* self;
 };
 
-// psi of the next step from the energy pass: have = d.psi already holds psi of this step (no
-// psi pass), want = the energy pass should write psi of the next step into d.psi_next; made is
-// set when it did.
+// psi of the next step: have = this step needs no psi pass (d.psi holds its psi, or the collision
+// makes it), want = the energy pass should see to that for the next step (by writing d.psi_next,
+// where the collision does not make psi); made is set when it did.
 struct PsiChain {
   int have, want, made;
 };

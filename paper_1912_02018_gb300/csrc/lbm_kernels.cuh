@@ -2,17 +2,16 @@
 // templated on the compute type C (double or float) and population storage type S.
 //
 // Layout: structure of arrays, every field [ny][pitch] with x fastest; populations are
-// 9 such planes, ping-ponged between two buffers.  The kernels:
+// 9 such planes, ping-ponged between two buffers.  Here: the building blocks, and the kernels of the
+// FP64 build and of FP16 population storage (their energy passes: lbm_energy_f64.cuh, one kernel
+// per Heun stage, and lbm_step_f16s.cuh).  The FP32 step: lbm_step_f32.cuh, lbm_flow_f32.cuh,
+// lbm_energy_f32.cuh.
 //   k_rho_psi pull f with boundary substitutions, rho, psi(rho, T); writes psi.  Runs only
-//             when no energy pass made psi (first step, after a restore, warm-up).
+//             when neither an energy pass made psi nor the collision makes it (first step,
+//             after a restore, warm-up).
 //   k_collide per 32x8 tile: the pull window of the 9 planes (1-node halo) and the psi tile
 //             (2-node halo) staged in shared memory by TMA (edge tiles: plain loads);
 //             interaction force, gravity, CM collision; writes f*, rho, u.
-//   k_energy  per 32x16 tile: T, rho, u staged by TMA with a 4-node halo, lambda(rho);
-//             Heun stage 1 on a 2-node halo, stage 2 on the tile, two nodes per thread;
-//             writes T^{n+1} and, from the pull of the new populations, psi of the next
-//             step; blocks holding wall nodes sum the wall heat flux in FP64 and the last
-//             block to finish adds the per-block partials in block order.
 //   kb_*      the same passes over the tiles of many domains in one launch per pass.
 // The operation order inside each node follows the paper's equations term by term so
 // that the FP64 build (compiled without FMA contraction) rounds like a plain reference;
@@ -362,6 +361,93 @@ __device__ __forceinline__ void grad_t(const C* p, int s, C& gx, C& gy) {
   gx = sx;
   gy = sy;
 }
+// ---------------------------------------------------------------- packed FP32 pairs and their stencils
+// The FP32 kernels handle two x-adjacent nodes per lane as one packed float2 (sm_100+ FFMA2, FADD2,
+// FMUL2: half the instructions, the same lane throughput).  Stencils fold a window row (columns
+// -2 .. 3 around the pair) into sums and differences over +/-1 and +/-2 columns, which every stencil
+// of the 25-point neighbourhood then takes its share of.
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.0f), a); }
+__device__ __forceinline__ float2 nabs2(float2 a) {
+  return make_float2(__uint_as_float(__float_as_uint(a.x) | 0x80000000u),
+                     __uint_as_float(__float_as_uint(a.y) | 0x80000000u));
+}
+__device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(rcp_approx(a.x), rcp_approx(a.y)); }
+
+// One window row of a column pair: the pair, and per node the difference and sum of its neighbours
+// at +/-1 (X1, S1) and +/-2 (X2, S2) columns.  q: the row's first window element (columns -2, -1).
+struct RowSums {
+  float2 c, X1, X2, S1, S2;
+};
+template <bool kX, bool kS>
+__device__ __forceinline__ RowSums row_sums(const float2* q) {
+  const float2 a = q[0], b = q[1], d = q[2];
+  RowSums r;
+  r.c = b;
+  if (kX) {
+    r.X1 = make_float2(__fsub_rn(b.y, a.y), __fsub_rn(d.x, b.x));
+    r.X2 = sub2(d, a);
+  }
+  if (kS) {
+    r.S1 = make_float2(__fadd_rn(b.y, a.y), __fadd_rn(d.x, b.x));
+    r.S2 = add2(d, a);
+  }
+  return r;
+}
+// Stencil weights by row distance k = |d|: of the pair (k, column offset 0, +/-1, +/-2).
+__device__ __forceinline__ constexpr float wrow(int k, int c) {
+  const int e = k * k + c * c;
+  return e == 1 ? float(4.0 / 21.0) : e == 2 ? float(4.0 / 45.0) : e == 4 ? float(1.0 / 60.0)
+       : e == 5 ? float(2.0 / 315.0) : e == 8 ? float(1.0 / 5040.0) : 0.0f;
+}
+// gx += the row's share of sum w e_x phi(x + e), at row distance k
+__device__ __forceinline__ void row_gx(const RowSums& r, int k, float2& gx) {
+  gx = fma2(f2(wrow(k, 1)), r.X1, fma2(f2(2.0f * wrow(k, 2)), r.X2, gx));
+}
+// gy += the row's share of sum w e_y phi(x + e), at row offset d != 0
+__device__ __forceinline__ void row_gy(const RowSums& r, int d, float2& gy) {
+  const int k = d < 0 ? -d : d;
+  gy = fma2(f2(d * wrow(k, 0)), r.c, fma2(f2(d * wrow(k, 1)), r.S1, fma2(f2(d * wrow(k, 2)), r.S2, gy)));
+}
+
+// The isotropic gradient of a column pair from the window rows -2 .. 2 (q: columns -2, -1 of the
+// middle row, row stride ts), and of one node from a 5x5 window (row-major, centre w[12]) with the
+// same roundings.  Rows are subtracted before they are weighted: exactly zero on a uniform field.
+__device__ __forceinline__ void grad_rows(const float2* q, int ts, float2& gx, float2& gy) {
+  gx = gy = f2(0.0f);
+  RowSums lo = row_sums<true, true>(q - 2 * ts), hi = row_sums<true, true>(q + 2 * ts);
+  row_gx(lo, 2, gx);
+  row_gx(hi, 2, gx);
+  gy = fma2(f2(2.0f * wrow(2, 0)), sub2(hi.c, lo.c),
+            fma2(f2(2.0f * wrow(2, 1)), sub2(hi.S1, lo.S1), fma2(f2(2.0f * wrow(2, 2)), sub2(hi.S2, lo.S2), gy)));
+  lo = row_sums<true, true>(q - ts);
+  hi = row_sums<true, true>(q + ts);
+  row_gx(lo, 1, gx);
+  row_gx(hi, 1, gx);
+  gy = fma2(f2(wrow(1, 0)), sub2(hi.c, lo.c),
+            fma2(f2(wrow(1, 1)), sub2(hi.S1, lo.S1), fma2(f2(wrow(1, 2)), sub2(hi.S2, lo.S2), gy)));
+  row_gx(row_sums<true, false>(q), 0, gx);
+}
+__device__ __forceinline__ void grad_window(const float* w, float& gx, float& gy) {
+  gx = gy = 0.0f;
+#pragma unroll
+  for (int k = 2; k >= 0; --k) {
+#pragma unroll
+    for (int t = 0; t < (k ? 2 : 1); ++t) {
+      const float* q = w + 5 * (t ? 2 + k : 2 - k);
+      gx = __fmaf_rn(wrow(k, 1), __fsub_rn(q[3], q[1]), __fmaf_rn(2.0f * wrow(k, 2), __fsub_rn(q[4], q[0]), gx));
+    }
+    if (k == 0) continue;
+    const float *a = w + 5 * (2 - k), *b = w + 5 * (2 + k);
+    gy = __fmaf_rn(k * wrow(k, 0), __fsub_rn(b[2], a[2]),
+                   __fmaf_rn(k * wrow(k, 1), __fsub_rn(__fadd_rn(b[3], b[1]), __fadd_rn(a[3], a[1])),
+                             __fmaf_rn(k * wrow(k, 2), __fsub_rn(__fadd_rn(b[4], b[0]), __fadd_rn(a[4], a[0])), gy)));
+  }
+}
+
 // ---------------------------------------------------------------- streaming (Sec. IV.A BCs)
 // Link fraction q of direction i at a near-wall node: the fraction of the link from the node
 // along -c_i that lies in the fluid (smallest root of |d + t c|^2 = r^2, tabulated at creation).
@@ -370,42 +456,36 @@ __device__ __forceinline__ C link_q(const Geo& g, int x, int y, int i) {
   return static_cast<const C*>(g.wall_q)[g.wall_idx[y * g.pitch + x] * 8 + i - 1];
 }
 
-// Pull with substitutions for nodes next to the wall, the inlet or the outlet: linear
-// interpolated bounce-back on the cylinder, Zou-He inlet, convective outlet.
-// side_out != nullptr: store the outlet's new streamed values there.
-template <typename C, typename S>
-__device__ __forceinline__ void pull_slow(const Geo& g, const Phys& ph, const S* __restrict__ f,
-                                          const uint8_t* __restrict__ mask, const C* __restrict__ side_in,
-                                          C* __restrict__ side_out, int x, int y, C fo[9]) {
+// Substitutions of the pull for nodes next to the wall, the inlet or the outlet, on the plainly pulled
+// fo: linear interpolated bounce-back on the cylinder, Zou-He inlet, convective outlet.  at(i, dx, dy):
+// population i at the node (x + dx, y + dy), |dx|, |dy| <= 1, inside the lattice.  The table of link
+// fractions tells which links meet the wall (no node types are read), so the loads of a node wait
+// for two others at most.  side_out != nullptr: store the outlet's new streamed values there.
+template <typename C, typename At>
+__device__ __forceinline__ void pull_special(const Geo& g, const Phys& ph, const C* __restrict__ side_in,
+                                             C* __restrict__ side_out, int x, int y, uint8_t m, C fo[9], const At& at) {
+  if (m & kNearWall) {
+    const C* wq = static_cast<const C*>(g.wall_q) + g.wall_idx[y * g.pitch + x] * 8 - 1;
+    C lq[9];
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const int cx = cxv(i), cy = cyv(i);
-    int sx = x - cx;
-    const int sy = wrap_y(g, y - cy);
-    if (g.periodic_x) sx = sx < 0 ? sx + g.nx : (sx >= g.nx ? sx - g.nx : sx);
-    C v;
-    if (sx < 0 || sx >= g.nx) {
-      v = C(0);  // unknown at the inlet or outlet; replaced below
-    } else if (mask[sy * g.pitch + sx] & kSolid) {
-      // linear interpolated bounce-back; the wall lies along c_opp(i)
+    for (int i = 1; i < 9; ++i) lq[i] = wq[i];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      // the wall lies along c_opp(i); its link fraction is -1 where the pull's source is fluid
       const int io = oppv(i);
-      const C q = link_q<C>(g, x, y, i);
-      const C a = ldf<C>(g, ph, f, io, y, x);
-      if (q < C(0.5)) {
-        int nxp = x + cx;
-        const int nyp = wrap_y(g, y + cy);
-        if (g.periodic_x) nxp = nxp < 0 ? nxp + g.nx : (nxp >= g.nx ? nxp - g.nx : nxp);
-        const bool ok = nxp >= 0 && nxp < g.nx && !(mask[nyp * g.pitch + nxp] & kSolid);
+      const C q = lq[i];
+      if (q >= C(0)) {
+        const C a = at(io, 0, 0);
         const C q2 = mul(C(2), q);
-        v = ok ? add(mul(q2, a), mul(sub(C(1), q2), ldf<C>(g, ph, f, io, nyp, nxp))) : a;
-      } else {
-        const C q2 = mul(C(2), q);
-        v = add(fdiv(a, q2), mul(fdiv(sub(q2, C(1)), q2), ldf<C>(g, ph, f, i, y, x)));
+        if (q < C(0.5)) {
+          const int nxp = x + cxv(i);
+          const bool ok = lq[io] < C(0) && (g.periodic_x || (nxp >= 0 && nxp < g.nx));
+          fo[i] = ok ? add(mul(q2, a), mul(sub(C(1), q2), at(io, cxv(i), cyv(i)))) : a;
+        } else {
+          fo[i] = add(fdiv(a, q2), mul(fdiv(sub(q2, C(1)), q2), at(i, 0, 0)));
+        }
       }
-    } else {
-      v = ldf<C>(g, ph, f, i, sy, sx);
     }
-    fo[i] = v;
   }
   if (g.periodic_x) return;
   if (x == 0) {
@@ -426,7 +506,7 @@ __device__ __forceinline__ void pull_slow(const Geo& g, const Phys& ph, const S*
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const int i = j == 0 ? 2 : (j == 1 ? 6 : 8);
-      const C inner = ldf<C>(g, ph, f, i, wrap_y(g, y - cyv(i)), g.nx - 1);
+      const C inner = at(i, 0, -cyv(i));
       const C s0 = side_in[j * g.ny + y];
       C v;
       if constexpr (sizeof(C) == 4) v = mad(pc<C>(ph).U_k, sub(inner, s0), s0);
@@ -434,6 +514,20 @@ __device__ __forceinline__ void pull_slow(const Geo& g, const Phys& ph, const S*
       fo[i] = v;
       if (side_out) side_out[j * g.ny + y] = v;
     }
+  }
+}
+
+// rho = sum_i f_i of pulled populations: in pairs of opposite directions in FP32 (whose moments use
+// the same sums), in the order of the index in FP64, as the reference does, and with FP16 storage.
+template <typename C, typename S>
+__device__ __forceinline__ C pop_sum(const C f[9]) {
+  if constexpr (sizeof(C) == 4 && sizeof(S) != 2) {
+    return add(add(f[0], add(add(f[1], f[2]), add(f[3], f[4]))), add(add(f[5], f[6]), add(f[7], f[8])));
+  } else {
+    C r = f[0];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) r = r + f[i];
+    return r;
   }
 }
 
@@ -463,7 +557,14 @@ __device__ __forceinline__ void pull_node(const Geo& g, const Phys& ph, const S*
   fo[7] = ldf<C>(g, ph, f, 7, yp, xm);
   fo[8] = ldf<C>(g, ph, f, 8, ym, xp);
   const bool edge = !g.periodic_x && (x == 0 || x == g.nx - 1);
-  if ((m & kNearWall) || edge) pull_slow<C, S>(g, ph, f, mask, side_in, side_out, x, y, fo);
+  if ((m & kNearWall) || edge) {
+    auto at = [&](int i, int dx, int dy) {
+      int sx = x + dx;
+      if (g.periodic_x) sx = sx < 0 ? sx + g.nx : (sx >= g.nx ? sx - g.nx : sx);
+      return ldf<C>(g, ph, f, i, wrap_y(g, y + dy), sx);
+    };
+    pull_special<C>(g, ph, side_in, side_out, x, y, m, fo, at);
+  }
 }
 
 // psi at node (x, y): pull, rho = sum f, Eq. (potential); solid nodes use rho_s.
@@ -474,12 +575,12 @@ __device__ __forceinline__ C psi_node(const Geo& g, const Phys& ph, const S* __r
   const int id = y * g.pitch + x;
   const uint8_t m = mask[id];
   const C t = T[id];
-  C fo[9];
-  pull_node<C, S>(g, ph, f, mask, side_in, nullptr, x, y, m, fo);
-  C rho = fo[0];
-#pragma unroll
-  for (int i = 1; i < 9; ++i) rho = rho + fo[i];
-  if (m & kSolid) rho = pc<C>(ph).rho_s;
+  C rho = pc<C>(ph).rho_s;
+  if (!(m & kSolid)) {
+    C fo[9];
+    pull_node<C, S>(g, ph, f, mask, side_in, nullptr, x, y, m, fo);
+    rho = pop_sum<C, S>(fo);
+  }
   return psi_of<C, PSI>(ph, rho, t, status);
 }
 
@@ -554,70 +655,6 @@ __device__ __forceinline__ void collide<double>(const double f[9], double rho, d
   fs[7] = diag(-q5, -0.25, 0.25);
   fs[8] = diag(-q5, 0.25, -0.25);
 }
-// The same for FP32 with every rounding written out (explicit fma, mul, add), so that the
-// result does not depend on which kernel inlines it.  Forward substitution of N(u) m* = k*
-// in closed form; m*_1 = k*_1 + u rho = m1 + Fx and m*_2 = m2 + Fy hold exactly since
-// u rho = m1 + Fx / 2.
-template <>
-__device__ __forceinline__ void collide<float>(const float f[9], float rho, float Fx, float Fy, float Fmx, float Fmy,
-                                               float psi, float omega, float sigma, float fs[9], float& ux,
-                                               float& uy) {
-  const float a56 = __fsub_rn(f[5], f[6]), a78 = __fsub_rn(f[7], f[8]);
-  const float m1 = __fadd_rn(__fadd_rn(__fsub_rn(f[1], f[2]), a56), a78);
-  const float m2 = __fsub_rn(__fadd_rn(__fsub_rn(f[3], f[4]), a56), a78);
-  const float m4 = __fsub_rn(__fadd_rn(f[1], f[2]), __fadd_rn(f[3], f[4]));
-  const float m5 = __fsub_rn(__fadd_rn(f[5], f[6]), __fadd_rn(f[7], f[8]));
-  const float u = __fdividef(__fmaf_rn(0.5f, Fx, m1), rho), v = __fdividef(__fmaf_rn(0.5f, Fy, m2), rho);
-  ux = u;
-  uy = v;
-  const float uu = __fmul_rn(u, u), vv = __fmul_rn(v, v), uv = __fmul_rn(u, v);
-  const float s2 = __fadd_rn(uu, vv), d2 = __fsub_rn(uu, vv), u2 = __fmul_rn(2.0f, u), v2 = __fmul_rn(2.0f, v);
-  // central moments k4, k5 of the pre-collision populations (Eq. (postColl2) shift)
-  const float k4 = __fmaf_rn(d2, rho, __fmaf_rn(v2, m2, __fmaf_rn(-u2, m1, m4)));
-  const float k5 = __fmaf_rn(uv, rho, __fmaf_rn(-v, m1, __fmaf_rn(-u, m2, m5)));
-  // post-collision central moments with the consistency terms alpha |Fm|^2
-  const float alpha = sigma != 0.0f ? __fdividef(sigma, __fmul_rn(psi, psi)) : 0.0f;
-  const float aF = __fmul_rn(alpha, __fmaf_rn(Fmx, Fmx, __fmul_rn(Fmy, Fmy)));
-  const float om = __fsub_rn(1.0f, omega);
-  const float ks3 = __fmaf_rn(2.0f, aF, __fmul_rn(2.0f / 3.0f, rho));
-  const float ks4 = __fmul_rn(om, k4), ks5 = __fmul_rn(om, k5);
-  const float ks6 = __fmul_rn(1.0f / 6.0f, Fy), ks7 = __fmul_rn(1.0f / 6.0f, Fx);
-  const float ks8 = __fmaf_rn(2.0f / 3.0f, aF, __fmul_rn(1.0f / 9.0f, rho));
-  // raw moments m* = N(u)^{-1} k*
-  const float ms1 = __fadd_rn(m1, Fx), ms2 = __fadd_rn(m2, Fy);
-  const float ms3 = __fmaf_rn(u2, ms1, __fmaf_rn(v2, ms2, __fmaf_rn(-s2, rho, ks3)));
-  const float ms4 = __fmaf_rn(u2, ms1, __fmaf_rn(-v2, ms2, __fmaf_rn(-d2, rho, ks4)));
-  const float ms5 = __fmaf_rn(v, ms1, __fmaf_rn(u, ms2, __fmaf_rn(-uv, rho, ks5)));
-  const float uv2 = __fmul_rn(2.0f, uv);
-  const float ms6 = __fmaf_rn(u2, ms5, __fmaf_rn(__fmul_rn(0.5f, v), __fadd_rn(ms3, ms4),
-                              __fmaf_rn(-uu, ms2, __fmaf_rn(-uv2, ms1, __fmaf_rn(__fmul_rn(uu, v), rho, ks6)))));
-  const float ms7 = __fmaf_rn(v2, ms5, __fmaf_rn(__fmul_rn(0.5f, u), __fsub_rn(ms3, ms4),
-                              __fmaf_rn(-uv2, ms2, __fmaf_rn(-vv, ms1, __fmaf_rn(__fmul_rn(u, vv), rho, ks7)))));
-  const float ms8 = __fmaf_rn(
-      u2, ms7,
-      __fmaf_rn(v2, ms6,
-                __fmaf_rn(__fmul_rn(-2.0f, uv2), ms5,
-                          __fmaf_rn(__fmul_rn(0.5f, d2), ms4,
-                                    __fmaf_rn(__fmul_rn(-0.5f, s2), ms3,
-                                              __fmaf_rn(__fmul_rn(uv2, u), ms2,
-                                                        __fmaf_rn(__fmul_rn(uv2, v), ms1,
-                                                                  __fmaf_rn(-__fmul_rn(uu, vv), rho, ks8))))))));
-  // f* = M^{-1} m*
-  const float A = __fmul_rn(0.25f, __fadd_rn(ms3, ms4)), B = __fmul_rn(0.25f, __fsub_rn(ms3, ms4));
-  const float c = __fmaf_rn(-0.5f, ms8, A), e = __fmaf_rn(-0.5f, ms8, B);
-  const float d = __fmul_rn(0.5f, __fsub_rn(ms1, ms7)), gy = __fmul_rn(0.5f, __fsub_rn(ms2, ms6));
-  fs[0] = __fadd_rn(__fsub_rn(rho, ms3), ms8);
-  fs[1] = __fadd_rn(c, d);
-  fs[2] = __fsub_rn(c, d);
-  fs[3] = __fadd_rn(e, gy);
-  fs[4] = __fsub_rn(e, gy);
-  const float sp = __fadd_rn(ms5, ms8), tp = __fadd_rn(ms6, ms7), wm = __fsub_rn(ms8, ms5), zm = __fsub_rn(ms6, ms7);
-  fs[5] = __fmul_rn(0.25f, __fadd_rn(sp, tp));
-  fs[6] = __fmul_rn(0.25f, __fsub_rn(sp, tp));
-  fs[7] = __fmul_rn(0.25f, __fsub_rn(wm, zm));
-  fs[8] = __fmul_rn(0.25f, __fadd_rn(wm, zm));
-}
-
 // Single-rate BGK on the same equilibrium and forcing, the operator the paper compares the CM
 // collision with (Sec. III.B): f* = f + omega (f^eq - f) + (1 - omega/2) F_i, u as above.  T(u) =
 // N(u) M is linear and maps f^eq and F_i to k^eq = (rho, 0, 0, 2 rho/3, 0, 0, 0, 0, rho/9) and
@@ -737,11 +774,15 @@ __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const
   const bool need_psi = multiphase && forcing;
   C fo[9];
   if (staged) {
-    // a staged tile holds no inlet or outlet column; wall nodes redo the pull with substitutions
 #pragma unroll
     for (int i = 0; i < 9; ++i)
       fo[i] = PopIO<C, S>::ld(s_f[(i * CS::FH + ty + 1 - cyv(i)) * CS::FW + tx + CS::XA - cxv(i)], i, ph);
-    if (m & kNearWall) pull_slow<C, S>(g, ph, f, mask, side_in, side_out, x, y, fo);
+    if (m & kNearWall) {  // a staged tile holds no edge column
+      const S* q = s_f + (ty + 1) * CS::FW + tx + CS::XA;
+      pull_special<C>(g, ph, side_in, side_out, x, y, m, fo, [&](int i, int dx, int dy) {
+        return PopIO<C, S>::ld(q[(i * CS::FH + dy) * CS::FW + dx], i, ph);
+      });
+    }
   } else {
     pull_node<C, S>(g, ph, f, mask, side_in, side_out, x, y, m, fo);
   }
@@ -846,9 +887,8 @@ __device__ __forceinline__ void collide_tile(const Geo& g, const Phys& ph, const
 }
 
 template <typename C, typename S, int OP = kCollCM>
-// FP32: at most 36 registers, so 7 blocks share an SM and more pulls are in flight (the pass
-// waits on DRAM: +10% over the default register budget; with FP16 storage 7 blocks and a few
-// spilled registers still beat 6 blocks without spills, 30.8 vs 32.6 us at 1536 x 768)
+// FP16 storage: at most 36 registers, so 7 blocks share an SM and more pulls are in flight (7 blocks
+// and a few spilled registers beat 6 without spills, 30.8 vs 32.6 us at 1536 x 768)
 __global__ void __launch_bounds__(kCollTX* kCollTY, sizeof(C) == 4 ? 7 : 1)
     k_collide(Geo g, Phys ph, const S* __restrict__ f, S* __restrict__ fn, const C* __restrict__ psi,
               const uint8_t* __restrict__ mask, const C* __restrict__ side_in, C* __restrict__ side_out,
@@ -933,176 +973,6 @@ __device__ __forceinline__ C lap_w(const C w[5][6], int c0) {
   }
   return C(2) * acc;
 }
-template <typename C>
-__device__ __forceinline__ C upwind3_w(const C w[5][6], int c0, bool along_x, C v) {
-  const C c = w[2][c0];
-  auto at = [&](int o) { return along_x ? w[2][c0 + o] : w[2 + o][c0]; };
-  if (v >= C(0)) {
-    C m2 = at(-2) - c, m1 = at(-1) - c, p1 = at(1) - c;
-    return fdiv(m2 - C(6) * m1 + C(2) * p1, C(6));
-  }
-  C m1 = at(-1) - c, p1 = at(1) - c, p2 = at(2) - c;
-  return fdiv(-C(2) * m1 + C(6) * p1 - p2, C(6));
-}
-// Eq. (energy) splits into parts that depend on rho and u only, frozen during the step
-// (lambda, grad lambda, div u), and parts that depend on the temperature being advanced.
-template <typename C>
-struct Frozen {
-  C lam0, lx, ly, divu;
-};
-// Frozen parts at the two nodes whose left one is at lam[0], u[0], v[0] (row stride as;
-// left node index even).
-template <typename C>
-__device__ __forceinline__ void frozen_pair(const C* lam, const C* u, const C* v, int as, Frozen<C> fz[2]) {
-  C w[5][6], unused, dxux[2], dyuy[2];
-  load_window(lam, as, w);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    fz[k].lam0 = w[2][2 + k];
-    grad_w(w, 2 + k, fz[k].lx, fz[k].ly);
-  }
-  load_window(u, as, w);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) grad_w<C, true, false>(w, 2 + k, dxux[k], unused);
-  load_window(v, as, w);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    grad_w<C, false, true>(w, 2 + k, unused, dyuy[k]);
-    fz[k].divu = dxux[k] + dyuy[k];
-  }
-}
-// Right-hand side at the same two nodes for the temperature tile t (row stride ts):
-// -u.grad T + (lambda lap T + grad lambda.grad T)/(rho c_v) - T (dp/dT)_rho div u / (rho c_v).
-template <typename C>
-__device__ __forceinline__ void energy_rhs_pair(const Phys& ph, const C* t, int ts, const C* u, const C* v,
-                                                const C* r, const Frozen<C> fz[2], C L[2]) {
-  C w[5][6];
-  load_window(t, ts, w);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const C u0 = u[k], v0 = v[k], T0 = w[2][2 + k], r0 = r[k];
-    C conv = u0 * upwind3_w(w, 2 + k, true, u0) + v0 * upwind3_w(w, 2 + k, false, v0);
-    C gx, gy;
-    grad_w(w, 2 + k, gx, gy);
-    C lap = lap_w(w, 2 + k);
-    C diff = fz[k].lam0 * lap + (fz[k].lx * gx + fz[k].ly * gy);
-    C work = T0 * dpdT_eos(ph, r0, T0) * fz[k].divu;
-    L[k] = -conv + fdiv(diff, r0 * pc<C>(ph).c_v) - fdiv(work, r0 * pc<C>(ph).c_v);
-  }
-}
-
-// FP32: the two nodes of a pair are one packed float2 throughout the stencil sums (sm_100+
-// FFMA2/FADD2/FMUL2), halving the FP32 instructions of the energy pass.  The window of a pair
-// is kept as aligned column pairs A[r][j] = (c_2j, c_2j+1) and shifted pairs B[r][j] =
-// (c_2j+1, c_2j+2); the value pair at offset ex is A[r][1 + ex/2] for even ex, B[r][(1 + ex)/2]
-// for odd ex.  Each packed operation rounds like the scalar one it replaces.
-struct Win2 {
-  float2 A[5][3], B[5][2];
-};
-__device__ __forceinline__ void load_win2(const float* p, int s, Win2& W) {
-#pragma unroll
-  for (int r = 0; r < 5; ++r) {
-    const float2* q = reinterpret_cast<const float2*>(p + (r - 2) * s - 2);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) W.A[r][c] = q[c];
-    W.B[r][0] = make_float2(W.A[r][0].y, W.A[r][1].x);
-    W.B[r][1] = make_float2(W.A[r][1].y, W.A[r][2].x);
-  }
-}
-__device__ __forceinline__ float2 win_at(const Win2& W, int r, int ex) {
-  return (ex & 1) ? W.B[r][(1 + ex) / 2] : W.A[r][1 + ex / 2];
-}
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-template <bool kX = true, bool kY = true>
-__device__ __forceinline__ void grad_w2(const Win2& W, float2& gx, float2& gy) {
-  float2 sx = f2(0.f), sy = f2(0.f);
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    const int ex = exv(k), ey = eyv(k);
-    if ((kX && ex != 0) || (kY && ey != 0)) {
-      const float2 d = sub2(win_at(W, 2 + ey, ex), win_at(W, 2 - ey, -ex));
-      if (kX && ex != 0) sx = __ffma2_rn(f2(float(wiso(k) * ex)), d, sx);
-      if (kY && ey != 0) sy = __ffma2_rn(f2(float(wiso(k) * ey)), d, sy);
-    }
-  }
-  gx = sx;
-  gy = sy;
-}
-__device__ __forceinline__ float2 lap_w2(const Win2& W) {
-  const float2 c = W.A[2][1];
-  float2 acc = f2(0.f);
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    const int ex = exv(k), ey = eyv(k);
-    const float2 d = __ffma2_rn(c, f2(-2.f), __fadd2_rn(win_at(W, 2 + ey, ex), win_at(W, 2 - ey, -ex)));
-    acc = __ffma2_rn(f2(float(wiso(k))), d, acc);
-  }
-  return __fmul2_rn(f2(2.f), acc);
-}
-// Six times the third-order upwind derivative of the pair along x (row 2) or y (column pair
-// 1), each node biased against the sign of its own velocity v.
-__device__ __forceinline__ float2 upwind6_w2(const Win2& W, bool along_x, float2 v) {
-  float2 q[5];
-#pragma unroll
-  for (int o = -2; o <= 2; ++o) q[o + 2] = along_x ? win_at(W, 2, o) : W.A[2 + o][1];
-  const float2 c = q[2];
-  const float2 m2 = sub2(q[0], c), m1 = sub2(q[1], c), p1 = sub2(q[3], c), p2 = sub2(q[4], c);
-  const float2 pos = __ffma2_rn(f2(2.f), p1, __ffma2_rn(f2(-6.f), m1, m2));
-  const float2 neg = sub2(__ffma2_rn(f2(6.f), p1, __fmul2_rn(f2(-2.f), m1)), p2);
-  return make_float2(v.x >= 0.f ? pos.x : neg.x, v.y >= 0.f ? pos.y : neg.y);
-}
-template <>
-__device__ __forceinline__ void frozen_pair<float>(const float* lam, const float* u, const float* v, int as,
-                                                   Frozen<float> fz[2]) {
-  Win2 W;
-  float2 lx, ly, dxux, dyuy, unused;
-  load_win2(lam, as, W);
-  fz[0].lam0 = W.A[2][1].x;
-  fz[1].lam0 = W.A[2][1].y;
-  grad_w2(W, lx, ly);
-  load_win2(u, as, W);
-  grad_w2<true, false>(W, dxux, unused);
-  load_win2(v, as, W);
-  grad_w2<false, true>(W, unused, dyuy);
-  const float2 dv = __fadd2_rn(dxux, dyuy);
-  fz[0].lx = lx.x, fz[0].ly = ly.x, fz[0].divu = dv.x;
-  fz[1].lx = lx.y, fz[1].ly = ly.y, fz[1].divu = dv.y;
-}
-__device__ __forceinline__ float2 pk_div(float2 a, float2 b) {
-  return make_float2(__fdividef(a.x, b.x), __fdividef(a.y, b.y));
-}
-template <>
-__device__ __forceinline__ void energy_rhs_pair<float>(const Phys& ph, const float* t, int ts, const float* u,
-                                                       const float* v, const float* r, const Frozen<float> fz[2],
-                                                       float L[2]) {
-  Win2 W;
-  load_win2(t, ts, W);
-  const float2 u2 = make_float2(u[0], u[1]), v2 = make_float2(v[0], v[1]);
-  const float2 conv6 = __ffma2_rn(u2, upwind6_w2(W, true, u2), __fmul2_rn(v2, upwind6_w2(W, false, v2)));
-  float2 gx, gy;
-  grad_w2(W, gx, gy);
-  const float2 lap = lap_w2(W);
-  const float2 diff = __ffma2_rn(make_float2(fz[0].lam0, fz[1].lam0), lap,
-                                 __ffma2_rn(make_float2(fz[0].lx, fz[1].lx), gx,
-                                            __fmul2_rn(make_float2(fz[0].ly, fz[1].ly), gy)));
-  // (dp/dT)_rho of Eq. (eos) with phi = (1 + kappa (1 - sqrt(T/Tc)))^2, dphi/dT = -kappa
-  // sqrt(phi) / sqrt(T Tc):  rep + att (kappa (1 + kappa) / sqrt(T Tc) - kappa^2 / Tc), with
-  // rep = rho R / (1 - b rho) and att = a rho^2 / (1 + 2 b rho - b^2 rho^2)
-  const PhysC<float>& k = ph.f;
-  const float2 rho = make_float2(r[0], r[1]), T0 = W.A[2][1];
-  const float2 rep = pk_div(__fmul2_rn(f2(k.R), rho), __ffma2_rn(f2(-k.b), rho, f2(1.0f)));
-  const float2 att = pk_div(__fmul2_rn(__fmul2_rn(f2(k.a), rho), rho),
-                            __ffma2_rn(rho, __ffma2_rn(f2(-k.b * k.b), rho, f2(2.0f * k.b)), f2(1.0f)));
-  const float2 rs = make_float2(rsqrtf(T0.x * k.Tc), rsqrtf(T0.y * k.Tc));
-  const float2 dpdT = __ffma2_rn(att, __ffma2_rn(f2(ph.dpdT_c1), rs, f2(-ph.dpdT_c2)), rep);
-  const float2 work = __fmul2_rn(__fmul2_rn(T0, dpdT), make_float2(fz[0].divu, fz[1].divu));
-  const float2 Lp = __ffma2_rn(sub2(diff, work), pk_div(f2(1.0f), __fmul2_rn(f2(k.c_v), rho)),
-                               __fmul2_rn(f2(-1.0f / 6.0f), conv6));
-  L[0] = Lp.x;
-  L[1] = Lp.y;
-}
-
 // Density of the pulled populations, rho = sum_i f*_i(x - c_i), at the nodes (x0, y) and
 // (x0 + 1, y), x0 even, for a pair none of whose pulls crosses the lattice edge or meets the
 // wall (1 <= x0, x0 + 2 <= nx - 1, 1 <= y <= ny - 2, no near-wall node): the planes with c_x = 0
@@ -1158,79 +1028,6 @@ __device__ __forceinline__ void pair_rho(const Geo& g, const Phys& ph, const S* 
   }
 }
 
-// Heun stage 2 at the pair whose left node is (x, y), T^{n+1} = (T + T1 + L(T1)) / 2, from
-// shared tiles: inputs sT, sL, sU, sV, sR, sM (row stride ax, pair at index a) and the stage-1
-// temperature sT1 (row stride bx, pair at index b); fz: the pair's frozen parts.  Nodes with
-// x >= nx or y >= ylim are skipped.  Writes T^{n+1}, T1 (t1_out) and, with FUSE and psi_out,
-// psi of the next step from the pull of the new populations fnew, side_new (Eq. potential);
-// adds the pair's wall heat flux -lambda grad T^n . n (Sec. IV.B) to q and sets mine when
-// the pair holds a near-wall node.
-template <typename C, typename S, int PSI, bool FUSE>
-__device__ __forceinline__ void stage2_pair(const Geo& g, const Phys& ph, const C* sT, const C* sL, const C* sU,
-                                            const C* sV, const C* sR, const uint8_t* sM, int ax, int a, const C* sT1,
-                                            int bx, int b, const Frozen<C>* fz_in, int x0, int y, int ylim,
-                                            C* __restrict__ Tout, C* __restrict__ t1_out, int do_hf,
-                                            const S* __restrict__ fnew, const uint8_t* __restrict__ mask,
-                                            const C* __restrict__ side_new, C* __restrict__ psi_out, int* status,
-                                            double& q, int& mine) {
-  const Frozen<C> fz[2] = {fz_in[0], fz_in[1]};
-  C L[2];
-  energy_rhs_pair(ph, &sT1[b], bx, &sU[a], &sV[a], &sR[a], fz, L);
-  C tnew[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const int x = x0 + k;
-    if (x < g.nx && y < ylim) {
-      C out;
-      if (sM[a + k] & kSolid) out = sT[a + k];
-      else if (!g.periodic_x && x == 0) out = pc<C>(ph).T_sat;
-      else out = ((sT[a + k] + sT1[b + k]) + L[k]) * C(0.5);
-      Tout[y * g.pitch + x] = out;
-      tnew[k] = out;
-      if (t1_out) t1_out[y * g.pitch + x] = sT1[b + k];  // the stage-1 temperature, for the adjoint
-      if (do_hf && (sM[a + k] & kNearWall)) {
-        C gx, gy;
-        grad_t(&sT[a + k], ax, gx, gy);
-        const double* nv = &g.wall_n[2 * g.wall_idx[y * g.pitch + x]];
-        q += -(double)sL[a + k] * ((double)gx * nv[0] + (double)gy * nv[1]);
-        mine = 1;
-      }
-    }
-  }
-  if constexpr (FUSE) {
-    if (psi_out) {
-      const uint8_t m0 = sM[a], m1 = sM[a + 1];
-      C r[2];
-      // a pair away from the wall, the open edges and the periodic seams pulls from one base
-      // address; the others take the general pull with its boundary substitutions
-      if (!((m0 | m1) & kNearWall) && y >= 1 && y + 1 < g.ny && x0 >= 1 && x0 + 3 <= g.nx) {
-        pair_rho<C, S>(g, ph, fnew, x0, y, r);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          r[k] = C(0);
-          if (x0 + k < g.nx && y < ylim) {
-            C fo[9];
-            pull_node<C, S>(g, ph, fnew, mask, side_new, nullptr, x0 + k, y, k ? m1 : m0, fo);
-            C t = fo[0];
-#pragma unroll
-            for (int i = 1; i < 9; ++i) t = t + fo[i];
-            r[k] = t;
-          }
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int x = x0 + k;
-        if (x < g.nx && y < ylim) {
-          const C rho = ((k ? m1 : m0) & kSolid) ? pc<C>(ph).rho_s : r[k];
-          psi_out[y * g.pitch + x] = psi_of<C, PSI>(ph, rho, tnew[k], status);
-        }
-      }
-    }
-  }
-}
-
 // Block-level end of the wall heat flux: FP64 block sums only in the blocks that hold wall
 // nodes (the others skip the fence and the counter); the last of those n_wall blocks to
 // finish adds all nblocks partials in block order (zero elsewhere), updates the running
@@ -1265,169 +1062,10 @@ __device__ __forceinline__ void heat_flux_blocks(double q, int mine, double* par
   }
 }
 
-template <typename C, int TY_ = (sizeof(C) == 8 ? 8 : kEnergyTY)>
-struct EnergyTile {
-  static constexpr int TX = kEnergyTX;
-  static constexpr int TY = TY_;          // FP64 defaults to 8 rows to keep shared memory under 48 KB
-  static constexpr int NT = TX * TY / 2;  // two nodes per thread
-};
-
-// Both Heun stages on tile (bx, by); bid, nblocks: this tile's index among the domain's
-// nblocks tiles (for the heat-flux partials and the last-block reduction).
-// With FUSE, and psi_out set, the tile also evaluates psi of the next step at its nodes: the
-// pull of the populations this step's collision wrote (fnew, side_new), rho their sum (rho_s
-// in the solid), T the new temperature (Eq. potential) -- the next step then needs no psi pass.
-// maps: tensor maps of the inputs, with which an interior tile stages them by TMA (else null:
-// plain loads); t1_out: where to store the stage-1 temperature (the adjoint's recompute).
-template <typename C, int ETY, typename S = C, int PSI = kPsiF64, bool FUSE = false>
-__device__ __forceinline__ void energy_tile(const Geo& g, const Phys& ph, const C* __restrict__ Tin,
-                                            C* __restrict__ Tout, const C* __restrict__ rho, const C* __restrict__ ux,
-                                            const C* __restrict__ uy, const uint8_t* __restrict__ mask,
-                                            double* partial, unsigned* counter, double* hf, int nb, int do_hf,
-                                            int n_wall_tiles, int bx, int by, int bid, int nblocks,
-                                            const S* __restrict__ fnew = nullptr, const C* __restrict__ side_new = nullptr,
-                                            C* __restrict__ psi_out = nullptr, int* status = nullptr,
-                                            C* __restrict__ t1_out = nullptr, const EnergyMaps* maps = nullptr,
-                                            bool starve = false) {
-  constexpr int TX = EnergyTile<C, ETY>::TX, TY = EnergyTile<C, ETY>::TY, NT = EnergyTile<C, ETY>::NT;
-  constexpr int H = 4, AX = TX + 2 * H, AY = TY + 2 * H;  // inputs: tile + 4
-  constexpr int BX = TX + 4, BY = TY + 4;                 // stage 1: tile + 2
-  static_assert(AX * AY * sizeof(C) % 128 == 0 && AX * sizeof(C) % 16 == 0, "TMA boxes of the input tile");
-  static_assert(AX % 4 == 0 && (AX * AY) % 4 == 0, "word-wise mask and float4 lambda staging");
-  __shared__ __align__(128) C sT[AY * AX];
-  __shared__ __align__(128) C sL[AY * AX];
-  __shared__ __align__(128) C sRUV[3 * AY * AX];  // rho, u_x, u_y: the planes of one TMA box
-  C* const sR = sRUV;
-  C* const sU = sRUV + AY * AX;
-  C* const sV = sRUV + 2 * AY * AX;
-  __shared__ uint64_t s_bar;
-  __shared__ __align__(16) C sT1[BY * BX];
-  __shared__ Frozen<C> sF[TX * TY];
-  __shared__ __align__(16) uint8_t sM[AY * AX];
-  __shared__ double red[NT / 32];
-  __shared__ int done_last;
-  const int tid = threadIdx.x;
-  const int x0 = bx * TX, y0 = by * TY;
-  const bool interior = x0 >= H && y0 >= H && x0 + TX + H <= g.nx && y0 + TY + H <= g.ny;
-  if (maps && interior) {
-    // the input boxes by TMA (T; rho, u_x, u_y in one 3-plane box; first column x0 - 4:
-    // 16-byte aligned); the mask with plain
-    // loads while they fly; lambda(rho) once rho has landed
-    if (tid == 0) tma::bar_init(&s_bar, 1);
-    __syncthreads();
-    if (tid == 0) {
-      tma::bar_expect_tx(&s_bar, 4 * AX * AY * sizeof(C));
-      // T comes from the energy pass before the previous kernel (the collision, which does not
-      // write it): its copy starts before that kernel ends; the test hook leaves the barrier
-      // armed with no copy issued
-      if (!starve) tma::load_2d(sT, &maps->T, &s_bar, x0 - H, y0 - H);
-    }
-    // the mask as 32-bit words (x0 - 4 and the row pitch are multiples of 4 bytes)
-    for (int p = tid; p < (AX / 4) * AY; p += NT) {
-      const int r = p / (AX / 4), c = p - r * (AX / 4);
-      reinterpret_cast<uint32_t*>(sM)[p] =
-          *reinterpret_cast<const uint32_t*>(mask + (y0 + r - H) * g.pitch + x0 - H + 4 * c);
-    }
-    pdl::wait();  // rho, u and the new populations are the collision's output
-    pdl::trigger();
-    if (tid == 0 && !starve) tma::load_3d(sRUV, &maps->ruv, &s_bar, x0 - H, y0 - H, 0);
-    const int tries = starve ? tma::kStarveTries : tma::kWaitTries;
-    const bool landed = tma::bar_wait(&s_bar, 0, tries);
-    if (__syncthreads_or(!landed)) {
-      // a copy did not land in time: report it, let the copies land (bounded) and stop the tile
-      // (a tile that holds wall nodes then misses its heat-flux partial; restoring a state with
-      // lbm_set_state resets that bookkeeping)
-      if (tid == 0) atomicOr(status, kStatusTimeoutEnergy);
-      tma::bar_wait(&s_bar, 0, tries);
-      return;
-    }
-    if constexpr (sizeof(C) == 4) {
-      for (int p = tid; p < AX * AY / 4; p += NT) {  // four nodes per thread
-        const float4 r4 = reinterpret_cast<const float4*>(sR)[p];
-        reinterpret_cast<float4*>(sL)[p] =
-            make_float4(lam_of(ph, r4.x), lam_of(ph, r4.y), lam_of(ph, r4.z), lam_of(ph, r4.w));
-      }
-    } else {
-      for (int p = tid; p < AX * AY; p += NT) sL[p] = lam_of(ph, sR[p]);
-    }
-  } else {
-    pdl::wait();
-    pdl::trigger();
-    for (int p = tid; p < AX * AY; p += NT) {
-      const int gx = x0 + p % AX - H, gy = y0 + p / AX - H;
-      const int nid = interior ? gy * g.pitch + gx : map_y(g, gy) * g.pitch + map_x(g, gx);
-      const C r = rho[nid];
-      sT[p] = Tin[nid];
-      sR[p] = r;
-      sL[p] = lam_of(ph, r);
-      sU[p] = ux[nid];
-      sV[p] = uy[nid];
-      sM[p] = mask[nid];
-    }
-  }
-  __syncthreads();
-  // stage 1: T1 = T + L(T) on the tile and a 2-node halo, two nodes per thread; the frozen
-  // parts of the tile's own nodes are kept for stage 2
-  for (int p = tid; p < (BX / 2) * BY; p += NT) {
-    const int by = p / (BX / 2), bx = (p % (BX / 2)) * 2;
-    const int a = (by + 2) * AX + bx + 2;
-    Frozen<C> fz[2];
-    frozen_pair(&sL[a], &sU[a], &sV[a], AX, fz);
-    C L[2];
-    energy_rhs_pair(ph, &sT[a], AX, &sU[a], &sV[a], &sR[a], fz, L);
-    const int tx = bx - 2, ty = by - 2;
-    if (tx >= 0 && tx < TX && ty >= 0 && ty < TY) {
-      sF[ty * TX + tx] = fz[0];
-      sF[ty * TX + tx + 1] = fz[1];
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int gx = x0 + bx + k - 2;
-      C t1;
-      if (sM[a + k] & kSolid) t1 = sT[a + k];  // solid nodes keep their wall temperature
-      else if (!g.periodic_x && gx == 0) t1 = pc<C>(ph).T_sat;
-      else t1 = sT[a + k] + L[k];
-      sT1[by * BX + bx + k] = t1;  // positions past a non-periodic edge are replaced below
-    }
-  }
-  __syncthreads();
-  if (!g.periodic_x && (x0 < 2 || x0 + TX + 2 > g.nx)) {
-    for (int p = tid; p < BX * BY; p += NT) {
-      const int bx = p % BX, by = p / BX;
-      const int gx = x0 + bx - 2;
-      if (gx < 0 || gx >= g.nx) sT1[p] = sT1[by * BX + (map_x(g, gx) - x0 + 2)];
-    }
-    __syncthreads();
-  }
-  // stage 2 on the tile: T^{n+1} = (T + T1 + L(T1)) / 2
-  const int tx = (tid % (TX / 2)) * 2, ty = tid / (TX / 2);
-  double q = 0.0;
-  int mine = 0;
-  stage2_pair<C, S, PSI, FUSE>(g, ph, sT, sL, sU, sV, sR, sM, AX, (ty + H) * AX + tx + H, sT1, BX,
-                               (ty + 2) * BX + tx + 2, &sF[ty * TX + tx], x0 + tx, y0 + ty, g.ny, Tout, t1_out, do_hf,
-                               fnew, mask, side_new, psi_out, status, q, mine);
-  if (do_hf) heat_flux_blocks<NT>(q, mine, partial, counter, n_wall_tiles, bid, nblocks, hf, nb, red, &done_last);
-}
-template <typename C, typename S, int PSI>
-// FP32: at most 51 registers, 5 blocks per SM (+2.5%); with FP16 storage 64 registers and
-// 4 blocks (the conversions of the fused psi pull need them: no spills)
-__global__ void __launch_bounds__(EnergyTile<C>::NT, sizeof(C) == 4 ? (sizeof(S) == 2 ? 4 : 5) : 1)
-    k_energy(Geo g, Phys ph, const C* __restrict__ Tin, C* __restrict__ Tout, const C* __restrict__ rho,
-             const C* __restrict__ ux, const C* __restrict__ uy, const uint8_t* __restrict__ mask,
-             double* partial, unsigned* counter, double* hf, int nb, int do_hf, int n_wall_tiles,
-             const S* __restrict__ fnew, const C* __restrict__ side_new, C* __restrict__ psi_out, int* status,
-             C* __restrict__ t1_out, const __grid_constant__ EnergyMaps maps, int flags) {
-  energy_tile<C, EnergyTile<C>::TY, S, PSI, true>(g, ph, Tin, Tout, rho, ux, uy, mask, partial, counter, hf, nb,
-                                                   do_hf, n_wall_tiles, blockIdx.x, blockIdx.y,
-                                                   blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y, fnew,
-                                                   side_new, psi_out, status, t1_out,
-                                                   (flags & kLaunchStaged) ? &maps : nullptr,
-                                                   (flags & kLaunchStarve) != 0);
-}
-
 }  // namespace kern
 }  // namespace lbm
 #include "lbm_energy_f64.cuh"
+#include "lbm_step_f16s.cuh"
 namespace lbm {
 namespace kern {
 
@@ -1479,7 +1117,7 @@ __global__ void __launch_bounds__(256) kb_rho_psi(const BatchDomain* __restrict_
 // A batched launch covers the blocks [block0, block0 + gridDim.x) of a pass, which belong to
 // the domains dom0 ..; their tensor maps come as kernel parameters (index k - dom0).
 template <typename C, typename S, int CTY>
-__global__ void __launch_bounds__(kCollTX* CTY, (sizeof(C) == 4 && CTY == 8) ? 7 : 1)
+__global__ void __launch_bounds__(kCollTX* CTY)
     kb_collide(const BatchDomain* __restrict__ doms, const int* __restrict__ map, int cur, long long step,
                int block0, int dom0, const __grid_constant__ CollLaunchMaps maps) {
   const int blk = block0 + blockIdx.x, k = map[blk];
@@ -1522,8 +1160,8 @@ static __global__ void __launch_bounds__(128)
   if (!D.energy || step < D.warmup) {
     // no energy update for this domain this step: carry T over so all domains flip together,
     // and make psi of the next state from the new populations and the unchanged T
-    for (int p = threadIdx.x; p < kEnergyTX * 8; p += 128) {
-      const int x = bx * kEnergyTX + p % kEnergyTX, y = by * 8 + p / kEnergyTX;
+    for (int p = threadIdx.x; p < kEnergyTX64 * 8; p += 128) {
+      const int x = bx * kEnergyTX64 + p % kEnergyTX64, y = by * 8 + p / kEnergyTX64;
       if (x < D.g.nx && y < D.g.ny) {
         Tout[y * D.g.pitch + x] = Tin[y * D.g.pitch + x];
         if (psi_next)
@@ -1538,43 +1176,6 @@ static __global__ void __launch_bounds__(128)
                static_cast<const double*>(D.d.ux), static_cast<const double*>(D.d.uy), D.d.mask, bx, by, fnew, side_new,
                psi_next, D.d.status);
 }
-template <typename C, int ETY, int PSI>
-// FP32: a register budget for 1280 threads per SM, as the single-domain energy pass
-__global__ void __launch_bounds__(EnergyTile<C, ETY>::NT, sizeof(C) == 4 ? 1280 / EnergyTile<C, ETY>::NT : 1) kb_energy(const BatchDomain* __restrict__ doms,
-                                                                   const int* __restrict__ map, int cur, int tcur,
-                                                                   long long step, int block0, int dom0,
-                                                                   const __grid_constant__ EnLaunchMaps maps) {
-  const int blk = block0 + blockIdx.x, k = map[blk];
-  const BatchDomain& D = doms[k];
-  const int local = blk - D.en_first, bx = local % D.en_ntx, by = local / D.en_ntx;
-  const C* Tin = static_cast<const C*>(D.d.T[tcur]);
-  C* Tout = static_cast<C*>(D.d.T[tcur ^ 1]);
-  const C* fnew = static_cast<const C*>(D.d.f[cur ^ 1]);
-  const C* side_new = static_cast<const C*>(D.d.side[cur ^ 1]);
-  C* psi_next = pc<C>(D.ph).G != C(0) ? psi_buf<C>(D, cur ^ 1) : nullptr;
-  if (!D.energy || step < D.warmup) {
-    // no energy update for this domain this step: carry T over so all domains flip together,
-    // and make psi of the next state from the new populations and the unchanged T
-    constexpr int TX = EnergyTile<C, ETY>::TX, TY = EnergyTile<C, ETY>::TY;
-    for (int p = threadIdx.x; p < TX * TY; p += EnergyTile<C, ETY>::NT) {
-      const int x = bx * TX + p % TX, y = by * TY + p / TX;
-      if (x < D.g.nx && y < D.g.ny) {
-        Tout[y * D.g.pitch + x] = Tin[y * D.g.pitch + x];
-        if (psi_next)
-          psi_next[y * D.g.pitch + x] =
-              psi_node<C, C, PSI>(D.g, D.ph, fnew, Tin, D.d.mask, side_new, x, y, D.d.status);
-      }
-    }
-    return;
-  }
-  const EnergyMaps* em = D.tma ? &maps.e[k - dom0] : nullptr;
-  energy_tile<C, ETY, C, PSI, true>(D.g, D.ph, Tin, Tout, static_cast<const C*>(D.d.rho),
-                                    static_cast<const C*>(D.d.ux), static_cast<const C*>(D.d.uy), D.d.mask,
-                                    D.d.partial, D.d.counter, D.d.hf, D.d.nb, D.d.nb > 0,
-                                    D.d.wall_tiles[ETY == 16 ? 1 : 0], bx, by, local, D.en_nblocks, fnew, side_new,
-                                    psi_next, D.d.status, nullptr, em);
-}
-
 template <typename C, typename S, int PSI, int CTY, int ETY>
 int batch_step_impl(const BatchDomain* doms, const int* map_psi, int nb_psi, const int* map_coll, int nb_coll,
                     const int* map_en, int nb_en, int cur, int tcur, long long step, int need_psi,
@@ -1600,14 +1201,11 @@ int batch_step_impl(const BatchDomain* doms, const int* map_psi, int nb_psi, con
     EnLaunchMaps m;
     for (int k = d0; k < d1; ++k) m.e[k - d0] = hmaps[k].em[tcur];
     const int b0 = hdoms[d0].en_first, b1 = d1 < ndom ? hdoms[d1].en_first : nb_en;
-    if constexpr (sizeof(C) == 8) kb_energy1_f64<<<b1 - b0, 128, 0, s>>>(doms, map_en, tcur, step, b0, d0, m);
-    else kb_energy<C, ETY, PSI><<<b1 - b0, EnergyTile<C, ETY>::NT, 0, s>>>(doms, map_en, cur, tcur, step, b0, d0, m);
+    kb_energy1_f64<<<b1 - b0, 128, 0, s>>>(doms, map_en, tcur, step, b0, d0, m);
     ++n;
   }
-  if constexpr (sizeof(C) == 8) {
-    kb_energy2_f64<<<nb_en, 128, 0, s>>>(doms, map_en, cur, tcur, step);
-    ++n;
-  }
+  kb_energy2_f64<<<nb_en, 128, 0, s>>>(doms, map_en, cur, tcur, step);
+  ++n;
   return cudaPeekAtLastError() == cudaSuccess ? n : -1;
 }
 
@@ -1617,16 +1215,15 @@ template <typename C, typename S>
 bool batch_maps_impl(BatchDomain& D, DomainMaps& m, int cty, int ety) {
   const Geo& g = D.g;
   const int XA = 16 / (int)sizeof(S), PA = 16 / (int)sizeof(C) < 2 ? 2 : 16 / (int)sizeof(C);
-  const int EH = sizeof(C) == 8 ? 4 : 8;  // both halos of the energy tile
   bool ok = D.d.tma != 0;
   for (int p = 0; p < 2 && ok; ++p) {
     ok = tma::encode<S>(&m.f[p], D.d.f[p], g.nx, g.ny, g.pitch, g.plane, 9, kCollTX + 2 * XA, cty + 2) &&
          tma::encode<C>(&m.psi[p], p ? D.d.psi_next : D.d.psi, g.nx, g.ny, g.pitch, g.plane, 1,
                         kCollTX + 2 * PA, cty + 4) &&
-         tma::encode<C>(&m.em[p].T, D.d.T[p], g.nx, g.ny, g.pitch, g.plane, 1, kEnergyTX + EH, ety + EH) &&
+         tma::encode<C>(&m.em[p].T, D.d.T[p], g.nx, g.ny, g.pitch, g.plane, 1, kEnergyTX64 + 4, ety + 4) &&
          static_cast<const C*>(D.d.ux) == static_cast<const C*>(D.d.rho) + g.plane &&
          static_cast<const C*>(D.d.uy) == static_cast<const C*>(D.d.rho) + 2 * (size_t)g.plane &&
-         tma::encode<C>(&m.em[p].ruv, D.d.rho, g.nx, g.ny, g.pitch, g.plane, 3, kEnergyTX + EH, ety + EH);
+         tma::encode<C>(&m.em[p].ruv, D.d.rho, g.nx, g.ny, g.pitch, g.plane, 3, kEnergyTX64 + 4, ety + 4);
   }
   D.tma = ok ? 1 : 0;
   return ok;
@@ -1737,11 +1334,20 @@ __global__ void k_export_force(Geo g, Phys ph, const C* __restrict__ psi, const 
 #pragma unroll
         for (int c = 0; c < 5; ++c) w[r * 5 + c] = psi[map_y(g, y + r - 2) * g.pitch + map_x(g, x + c - 2)];
       C sx, sy;
-      grad_t(&w[12], 5, sx, sy);
-      Fmx = -k.G * cs2 * w[12] * sx;
-      Fmy = -k.G * cs2 * w[12] * sy;
+      if constexpr (sizeof(C) == 4) {
+        grad_window(w, sx, sy);
+        const C a = mul(ph.sc.gm, w[12]);
+        Fmx = mul(a, sx);
+        Fmy = mul(a, sy);
+      } else {
+        grad_t(&w[12], 5, sx, sy);
+        Fmx = -k.G * cs2 * w[12] * sx;
+        Fmy = -k.G * cs2 * w[12] * sy;
+      }
     }
-    C Fx = sub(Fmx, mul(sub(rho[id], k.rho_l), k.g));
+    C Fx;
+    if constexpr (sizeof(C) == 4) Fx = mad(-k.g, sub(rho[id], k.rho_l), Fmx);
+    else Fx = sub(Fmx, mul(sub(rho[id], k.rho_l), k.g));
     if (k.body_fx != C(0)) Fx = add(Fx, k.body_fx);
     out = comp == 0 ? (double)Fx : (double)Fmy;
   }
@@ -1844,29 +1450,28 @@ int step_impl(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int
     const int do_hf = d.nb > 0;
     const bool fuse = chain && chain->want && ph.d.G != 0.0;
     pre(kKEnergy);
-    using ET = EnergyTile<C>;
-    const dim3 blk(ET::NT), grd((g.nx + ET::TX - 1) / ET::TX, (g.ny + ET::TY - 1) / ET::TY);
-    constexpr int EH = sizeof(C) == 8 ? 4 : 8;  // both halos
-    constexpr int AX = ET::TX + EH, AY = ET::TY + EH;
+    constexpr bool f64 = sizeof(C) == 8;
+    constexpr int TY = f64 ? 8 : EnergyTile16::TY, EH = f64 ? 4 : 8;  // both halos of the tile
+    const dim3 blk(kEnergyTX64 * TY / 2), grd((g.nx + kEnergyTX64 - 1) / kEnergyTX64, (g.ny + TY - 1) / TY);
+    constexpr int AX = kEnergyTX64 + EH, AY = TY + EH;
     EnergyMaps em;
     const bool ruv = ux == rho + g.plane && uy == rho + 2 * (size_t)g.plane;  // consecutive planes
     const bool e_staged = d.tma && ruv && tma::encode<C>(&em.T, T, g.nx, g.ny, g.pitch, g.plane, 1, AX, AY) &&
                           tma::encode<C>(&em.ruv, rho, g.nx, g.ny, g.pitch, g.plane, 3, AX, AY);
     const int eflags = e_staged ? (kLaunchStaged | ((d.starve & kStarveEnergy) ? kLaunchStarve : 0)) : 0;
-    if constexpr (sizeof(C) == 8) {
+    if constexpr (f64) {
       double* en64 = static_cast<double*>(d.en64);
       double* T1 = d.t1_out ? static_cast<double*>(d.t1_out) : en64;
-      launch_dep(d.pdl, grd, blk, 0, s, k_energy1_f64, g, ph, T, T1, en64, lam, rho, ux, uy, d.mask, d.partial, d.counter,
-                 d.hf, d.nb, do_hf, d.wall_tiles[0], d.status, em, eflags);
+      launch_dep(d.pdl, grd, blk, 0, s, k_energy1_f64, g, ph, T, T1, en64, lam, rho, ux, uy, d.mask, d.partial,
+                 d.counter, d.hf, d.nb, do_hf, d.wall_tiles[0], d.status, em, eflags);
       launch_dep(d.pdl, grd, blk, 0, s, k_energy2_f64, g, ph, T, Tn, T1, en64, lam, rho, ux, uy, d.mask,
                  fuse ? static_cast<const double*>(fn) : nullptr, side_out,
                  fuse ? static_cast<double*>(d.psi_next) : nullptr, d.status);
       ++n;
     } else {
-      launch_dep(d.pdl, grd, blk, 0, s, k_energy<C, S, PSI>, g, ph, T, Tn, rho, ux, uy, d.mask, d.partial, d.counter,
-                 d.hf, d.nb, do_hf, d.wall_tiles[ET::TY == 16 ? 1 : 0], fuse ? static_cast<const S*>(fn) : nullptr,
-                 static_cast<const C*>(side_out), fuse ? static_cast<C*>(d.psi_next) : nullptr, d.status,
-                 static_cast<C*>(d.t1_out), em,
+      launch_dep(d.pdl, grd, blk, 0, s, k_energy_f16s<PSI>, g, ph, T, Tn, rho, ux, uy, d.mask, d.partial, d.counter,
+                 d.hf, d.nb, do_hf, d.wall_tiles[1], fuse ? static_cast<const __half*>(fn) : nullptr,
+                 static_cast<const float*>(side_out), fuse ? static_cast<float*>(d.psi_next) : nullptr, d.status, em,
                  eflags);
     }
     post(kKEnergy);
