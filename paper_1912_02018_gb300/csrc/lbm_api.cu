@@ -1100,7 +1100,8 @@ static int batch_launch(lbm_batch* b, cudaStream_t s) {
                                       b->h_doms.data(), b->hmaps.data(), nd, s);
 }
 
-// After a batched step: the energy pass has made psi of the new state in buffer b->cur; each
+// After a batched step: the energy pass has made psi of the new state in buffer b->cur (FP64; the
+// FP32 collision makes psi itself); each
 // domain's context sees the buffers as a single-domain step leaves them (psi: the one the
 // step's collision used, psi_next: the pending one)
 static void batch_advance(lbm_batch* b, int launches) {

@@ -135,8 +135,8 @@ struct BatchDomain {
   long long warmup;
   int energy;
   int psi_first, psi_ntx;                 // psi pass: 32 x 8 tiles
-  int coll_first, coll_ntx;               // collision pass: 32 x CTY tiles
-  int en_first, en_ntx, en_nblocks;       // energy pass: 32 x ETY tiles
+  int coll_first, coll_ntx;               // collision pass: 32 (FP64) or 60 x CTY tiles
+  int en_first, en_ntx, en_nblocks;       // energy pass: 32 (FP64) or 60 x ETY tiles
   int tma;                                // 1: the launch passes this domain's tensor maps
 };
 
