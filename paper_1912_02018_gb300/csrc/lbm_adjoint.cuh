@@ -22,50 +22,37 @@ namespace adj {
 
 using namespace kern;
 
-// ---------------------------------------------------------------- dual numbers
+// ---------------------------------------------------------------- derivatives of the equation of state
+// Closed forms for Eq. (eos), p = R T rho / (1 - b rho) - a phi(T) rho^2 / D, D = 1 + 2 b rho - b^2 rho^2,
+// phi = s^2, s = 1 + kappa (1 - sqrt(T / Tc)):  with h = 1 / sqrt(T Tc), ds/dT = -kappa h / 2,
+// dphi/dT = -kappa s h, d2phi/dT2 = kappa h^2 (kappa + s h Tc) / 2, and d(rho^2 / D)/d rho = 2 rho (1 + b rho) / D^2.
+// Three quotients and a root a node; forward-mode dual numbers, which these replace, took up to sixteen quotients,
+// and a quotient or root costs about ten operations of the FP64 pipe that bounds the FP64 window.
+// With the one reciprocal of rho c_v or rho a node in k_adj_energy and k_adj_collide, constant factors instead of
+// constant divisors, and no products with zero stencil coefficients: a 100-step FP64 window on 256 x 128 52.5 -> 42.1 ms,
+// a 250-step FP32 window on 512 x 256 26.4 -> 25.9 ms.  The FP32 reverse kernels are bound by the latency of a block, not
+// by issue: 448 threads a block in the energy stages (a tile's sources in one round) gave 26.2 ms, dependent launches
+// with the forward-only work ahead of the wait 25.8 ms, and 47.3 ms in FP64.
 template <typename C>
-struct Dl {
-  C v, d;
+struct EosD {
+  C dpdT, dpdT_T, dpdT_r;  // dp/dT and its derivatives with respect to T and rho
+  C dpdr;                  // dp/d rho
 };
 template <typename C>
-__device__ __forceinline__ Dl<C> operator+(Dl<C> a, Dl<C> b) { return {a.v + b.v, a.d + b.d}; }
-template <typename C>
-__device__ __forceinline__ Dl<C> operator-(Dl<C> a, Dl<C> b) { return {a.v - b.v, a.d - b.d}; }
-template <typename C>
-__device__ __forceinline__ Dl<C> operator*(Dl<C> a, Dl<C> b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
-template <typename C>
-__device__ __forceinline__ Dl<C> operator/(Dl<C> a, Dl<C> b) {
-  const C q = fdiv(a.v, b.v);
-  return {q, fdiv(a.d - q * b.d, b.v)};
-}
-template <typename C>
-__device__ __forceinline__ Dl<C> operator*(C s, Dl<C> a) { return {s * a.v, s * a.d}; }
-template <typename C>
-__device__ __forceinline__ Dl<C> operator+(C s, Dl<C> a) { return {s + a.v, a.d}; }
-template <typename C>
-__device__ __forceinline__ Dl<C> operator-(C s, Dl<C> a) { return {s - a.v, -a.d}; }
-template <typename C>
-__device__ __forceinline__ Dl<C> dsqrt(Dl<C> a) {
-  const C s = sqrt(a.v);
-  return {s, fdiv(a.d, C(2) * s)};
-}
-
-// Peng-Robinson p(rho, T), Eq. (eos), and (dp/dT)_rho, on dual numbers.
-template <typename C>
-__device__ __forceinline__ Dl<C> pr_p(const PhysC<C>& k, Dl<C> rho, Dl<C> T) {
-  const Dl<C> s = C(1) + k.kappa * (C(1) - dsqrt(T * Dl<C>{C(1) / k.Tc, C(0)}));
-  const Dl<C> rep = (k.R * T) * rho / (C(1) - k.b * rho);
-  const Dl<C> att = (k.a * (s * s)) * (rho * rho) / ((C(1) + C(2) * k.b * rho) - (k.b * k.b) * (rho * rho));
-  return rep - att;
-}
-template <typename C>
-__device__ __forceinline__ Dl<C> pr_dpdT(const PhysC<C>& k, Dl<C> rho, Dl<C> T) {
-  const Dl<C> sq = dsqrt(T * Dl<C>{C(1) / k.Tc, C(0)});
-  const Dl<C> s = C(1) + k.kappa * (C(1) - sq);
-  const Dl<C> dphi = (-k.kappa * s) / dsqrt(T * Dl<C>{k.Tc, C(0)});
-  const Dl<C> rep = k.R * rho / (C(1) - k.b * rho);
-  const Dl<C> att = (k.a * dphi) * (rho * rho) / ((C(1) + C(2) * k.b * rho) - (k.b * k.b) * (rho * rho));
-  return rep - att;
+__device__ __forceinline__ EosD<C> eos_d(const PhysC<C>& k, C rho, C T) {
+  const C h = fdiv(C(1), sqrt(T * k.Tc));
+  const C s = C(1) + k.kappa * (C(1) - T * h);  // T h = sqrt(T / Tc)
+  const C i1 = fdiv(C(1), C(1) - k.b * rho);
+  const C iD = fdiv(C(1), (C(1) + C(2) * k.b * rho) - (k.b * k.b) * (rho * rho));
+  const C att = k.a * (rho * rho) * iD;                                 // a rho^2 / D
+  const C attr = (C(2) * k.a) * (rho * (C(1) + k.b * rho)) * (iD * iD);  // its derivative
+  const C kh = k.kappa * h, dphi = -kh * s;
+  EosD<C> e;
+  e.dpdT = k.R * rho * i1 - att * dphi;
+  e.dpdT_T = -att * (C(0.5) * kh * (kh + s * (h * h) * k.Tc));
+  e.dpdT_r = k.R * (i1 * i1) - attr * dphi;
+  e.dpdr = k.R * T * (i1 * i1) - attr * (s * s);
+  return e;
 }
 // d phase_frac / d rho with the branch of the clamp that the forward took (inclusive ends).
 template <typename C>
@@ -136,7 +123,7 @@ struct Parts {
 };
 template <typename C>
 __device__ __forceinline__ C upwind_d(C m2, C m1, C p1, C p2, C v) {
-  return v >= C(0) ? fdiv(m2 - C(6) * m1 + C(2) * p1, C(6)) : fdiv(-C(2) * m1 + C(6) * p1 - p2, C(6));
+  return (v >= C(0) ? m2 - C(6) * m1 + C(2) * p1 : -C(2) * m1 + C(6) * p1 - p2) * C(1.0 / 6.0);
 }
 template <typename C>
 __device__ __forceinline__ Parts<C> parts_at(const C* t, int ts, const C* l, const C* u, const C* v, int as) {
@@ -237,12 +224,12 @@ __global__ void __launch_bounds__(kEANT) k_adj_energy(Args<C> a) {
         const Parts<C> P = parts_at(t, ts, &sL[ai], &sU[ai], &sV[ai], AX);
         const C r0 = sR[ai], T0 = t[0], lam0 = sL[ai];
         const C rc = r0 * k.c_v;
-        const Dl<C> dT = pr_dpdT(k, Dl<C>{r0, C(0)}, Dl<C>{T0, C(1)});
-        const Dl<C> dR = pr_dpdT(k, Dl<C>{r0, C(1)}, Dl<C>{T0, C(0)});
+        const C irc = fdiv(C(1), rc), sr = s * irc;  // one quotient for all terms over rho c_v
+        const EosD<C> e = eos_d(k, r0, T0);
         const C diff = lam0 * P.lap + (P.lx * P.gx + P.ly * P.gy);
-        const C work = T0 * dT.v * P.divu;
-        C p1 = s * fdiv(P.lx, rc), p2 = s * fdiv(P.ly, rc);
-        C llam = s * fdiv(P.lap, rc);
+        const C work = T0 * e.dpdT * P.divu;
+        C p1 = sr * P.lx, p2 = sr * P.ly;
+        C llam = sr * P.lap;
         if (hf) {
           // q = -lambda grad T . n at this boundary node (Sec. IV.B)
           const double* nv = &g.wall_n[2 * g.wall_idx[gid]];
@@ -251,19 +238,20 @@ __global__ void __launch_bounds__(kEANT) k_adj_energy(Args<C> a) {
           p2 = p2 - a.wq * lam0 * nyv;
           llam = llam - a.wq * (P.gx * nxv + P.gy * nyv);
         }
-        Pv[0] = s * fdiv(lam0, rc);
+        Pv[0] = sr * lam0;
         Pv[1] = p1;
         Pv[2] = p2;
         Pv[3] = s * sU[ai];
         Pv[4] = s * sV[ai];
-        Pv[5] = -s * fdiv(T0 * dT.v, rc);
-        Pv[6] = s * fdiv(P.gx, rc);
-        Pv[7] = s * fdiv(P.gy, rc);
-        Lv[0] = -s * fdiv(P.divu, rc) * (dT.v + T0 * dT.d);
+        Pv[5] = -sr * (T0 * e.dpdT);
+        Pv[6] = sr * P.gx;
+        Pv[7] = sr * P.gy;
+        Lv[0] = -sr * P.divu * (e.dpdT + T0 * e.dpdT_T);
         Lv[1] = -s * P.upx;
         Lv[2] = -s * P.upy;
         Lv[3] = llam;
-        Lv[4] = s * (-fdiv(diff - work, rc * r0) - fdiv(T0 * P.divu * dR.d, rc));
+        // 1 / (rho^2 c_v) = irc^2 c_v
+        Lv[4] = -sr * ((diff - work) * (irc * k.c_v) + T0 * P.divu * e.dpdT_r);
       }
     }
 #pragma unroll
@@ -290,11 +278,17 @@ __global__ void __launch_bounds__(kEANT) k_adj_energy(Args<C> a) {
       const C w = C(w_of(ex, ey));
       const C clap = (ex == 0 && ey == 0) ? C(-4) * wsum : C(2) * w;
       tb = tb + clap * sP[pp];
-      if (ex != 0 || ey != 0) {
-        tb = tb + w * (C(ex) * sP[PN + pp] + C(ey) * sP[2 * PN + pp]);
-        ubx = ubx + w * C(ex) * sP[5 * PN + pp];
-        uby = uby + w * C(ey) * sP[5 * PN + pp];
-        lb = lb + w * (C(ex) * sP[6 * PN + pp] + C(ey) * sP[7 * PN + pp]);
+      // one product per non-zero coefficient: the compiler may not drop a product with zero
+      const C wx = w * C(ex), wy = w * C(ey);
+      if (ex != 0) {
+        tb = tb + wx * sP[PN + pp];
+        ubx = ubx + wx * sP[5 * PN + pp];
+        lb = lb + wx * sP[6 * PN + pp];
+      }
+      if (ey != 0) {
+        tb = tb + wy * sP[2 * PN + pp];
+        uby = uby + wy * sP[5 * PN + pp];
+        lb = lb + wy * sP[7 * PN + pp];
       }
       if (ey == 0) tb = tb - upw_coef<C>(ex, sU[ap] >= C(0)) * sP[3 * PN + pp];
       if (ex == 0) tb = tb - upw_coef<C>(ey, sV[ap] >= C(0)) * sP[4 * PN + pp];
@@ -375,30 +369,32 @@ __global__ void __launch_bounds__(256) k_adj_collide(Args<C> a) {
     for (int kk = 0; kk < 12; ++kk) {
       const int ex = exv(kk), ey = eyv(kk);
       const C d = at(g, a.psi, x + ex, y + ey) - at(g, a.psi, x - ex, y - ey);
-      sx = sx + C(wiso(kk)) * d * C(ex);
-      sy = sy + C(wiso(kk)) * d * C(ey);
+      if (ex != 0) sx = sx + C(wiso(kk) * ex) * d;
+      if (ey != 0) sy = sy + C(wiso(kk) * ey) * d;
     }
     Fmx = -k.G * cs2 * psi0 * sx;
     Fmy = -k.G * cs2 * psi0 * sy;
   }
   const C Fx = Fmx - (rho - k.rho_l) * k.g, Fy = Fmy;
   const C nu = nu_of(a.ph, rho);
-  const C omega = fdiv(C(1), fdiv(nu, cs2) + C(0.5));
+  const C omega = fdiv(C(1), C(3) * nu + C(0.5));
+  const C ir = fdiv(C(1), rho), third = C(1.0 / 3.0), sixth = C(1.0 / 6.0);  // one quotient for all terms over rho
   const C sig = multiphase ? k.sigma : C(0);
   const C m1 = ((((fo[1] - fo[2]) + fo[5]) - fo[6]) + fo[7]) - fo[8];
   const C m2 = ((((fo[3] - fo[4]) + fo[5]) - fo[6]) - fo[7]) + fo[8];
   const C m4 = ((fo[1] + fo[2]) - fo[3]) - fo[4];
   const C m5 = ((fo[5] + fo[6]) - fo[7]) - fo[8];
-  const C u = fdiv(m1 + C(0.5) * Fx, rho), v = fdiv(m2 + C(0.5) * Fy, rho);
+  const C u = (m1 + C(0.5) * Fx) * ir, v = (m2 + C(0.5) * Fy) * ir;
   const C k4 = (((u * u - v * v) * rho - C(2) * u * m1) + C(2) * v * m2) + m4;
   const C k5 = (((u * v) * rho - v * m1) - u * m2) + m5;
-  const C alpha = sig != C(0) ? fdiv(sig, psi0 * psi0) : C(0);
+  const C ipsi = sig != C(0) ? fdiv(C(1), psi0) : C(0);
+  const C alpha = sig * (ipsi * ipsi);
   const C Fm2 = Fmx * Fmx + Fmy * Fmy;
   // post-collision central moments k*
   const C K0 = rho, K1 = C(0.5) * Fx, K2 = C(0.5) * Fy;
-  const C K3 = fdiv(C(2) * rho, C(3)) + C(2) * alpha * Fm2;
+  const C K3 = C(2) * third * rho + C(2) * alpha * Fm2;
   const C K4 = (C(1) - omega) * k4, K5 = (C(1) - omega) * k5;
-  const C K6 = fdiv(Fy, C(6)), K7 = fdiv(Fx, C(6));
+  const C K6 = Fy * sixth, K7 = Fx * sixth;
   // seeds on f*; m*-bar = M^{-T} f*-bar (closed form of M^{-1})
   C fb[9];
 #pragma unroll
@@ -438,11 +434,11 @@ __global__ void __launch_bounds__(256) k_adj_collide(Args<C> a) {
            b8 * (C(2) * uu * v * K0 + C(4) * uv * K1 + C(2) * uu * K2 + v * K3 + v * K4 + C(4) * u * K5 +
                  C(2) * K6);
   // k* -> rho, F, alpha |F_m|^2, k4, k5, omega
-  C rb = kb0 + fdiv(C(2) * kb3, C(3)) + fdiv(kb8, C(9));
-  C Fbx = h * kb1 + fdiv(kb7, C(6)), Fby = h * kb2 + fdiv(kb6, C(6));
-  const C Abar = C(2) * kb3 + fdiv(C(2) * kb8, C(3));
+  C rb = kb0 + C(2) * third * kb3 + C(1.0 / 9.0) * kb8;
+  C Fbx = h * kb1 + sixth * kb7, Fby = h * kb2 + sixth * kb6;
+  const C Abar = C(2) * kb3 + C(2) * third * kb8;
   C Fmbx = Abar * alpha * C(2) * Fmx, Fmby = Abar * alpha * C(2) * Fmy;
-  const C psib = sig != C(0) ? Abar * Fm2 * fdiv(C(-2) * sig, psi0 * psi0 * psi0) : C(0);
+  const C psib = Abar * Fm2 * (C(-2) * alpha * ipsi);
   const C k4b = (C(1) - omega) * kb4, k5b = (C(1) - omega) * kb5;
   const C omb = -(k4 * kb4 + k5 * kb5);
   C mb0 = (uu - vv) * k4b + uv * k5b;
@@ -455,13 +451,14 @@ __global__ void __launch_bounds__(256) k_adj_collide(Args<C> a) {
   ubar = ubar + a.ub[0][id];
   vbar = vbar + a.ub[1][id];
   // u = (m1 + F/2) / rho
-  mb1 = mb1 + fdiv(ubar, rho);
-  mb2 = mb2 + fdiv(vbar, rho);
-  Fbx = Fbx + fdiv(ubar, C(2) * rho);
-  Fby = Fby + fdiv(vbar, C(2) * rho);
-  rb = rb - fdiv(u * ubar + v * vbar, rho);
+  const C ur = ubar * ir, vr = vbar * ir;
+  mb1 = mb1 + ur;
+  mb2 = mb2 + vr;
+  Fbx = Fbx + h * ur;
+  Fby = Fby + h * vr;
+  rb = rb - (u * ur + v * vr);
   // omega = 1 / (nu(rho)/cs^2 + 1/2)
-  rb = rb - omb * omega * omega * fdiv(dphase(k, rho) * (k.nu_l - k.nu_v), cs2);
+  rb = rb - omb * omega * omega * (C(3) * (dphase(k, rho) * (k.nu_l - k.nu_v)));
   // F = F_m + gravity
   Fmbx = Fmbx + Fbx;
   Fmby = Fmby + Fby;
@@ -518,8 +515,10 @@ __global__ void __launch_bounds__(256) k_adj_force(Args<C> a) {
       grad_t(&sPsi[c], HX, sx, sy);
       pb = pb + gc * (sFx[c] * sx + sFy[c] * sy);
     }
+    C pn = C(0);
     auto add = [&](int ex, int ey, int s) {
-      pb = pb + gc * sPsi[s] * C(w_of(ex, ey)) * (C(ex) * sFx[s] + C(ey) * sFy[s]);
+      const C wx = C(w_of(ex, ey)) * C(ex), wy = C(w_of(ex, ey)) * C(ey);
+      pn = pn + sPsi[s] * (ey == 0 ? wx * sFx[s] : ex == 0 ? wy * sFy[s] : wx * sFx[s] + wy * sFy[s]);
     };
     if (g.periodic_x || (x > 0 && x < g.nx - 1)) {
       // one source position per offset (ghost positions carry no F_m adjoint)
@@ -539,14 +538,14 @@ __global__ void __launch_bounds__(256) k_adj_force(Args<C> a) {
           for (int sx = lo; sx <= hi; ++sx) add(ex, ey, (ty + 2 - ey) * HX + sx - x0 + 2);
         }
     }
+    pb = pb + gc * pn;
     // psi = sqrt(rad), rad = k2 (p - rho cs^2), k2 = 2 / (G cs^2)
     const C r0 = a.rho[id], T0 = a.T[id], psi0 = sPsi[c];
     const C k2 = fdiv(C(2), k.G * cs2);
-    const C dpr = pr_p(k, Dl<C>{r0, C(1)}, Dl<C>{T0, C(0)}).d;
-    const C dpt = dpdT_eos(a.ph, r0, T0);
+    const EosD<C> e = eos_d(k, r0, T0);
     const C inv2psi = fdiv(C(1), C(2) * psi0);
-    if (!(m & kSolid)) rp = pb * k2 * (dpr - cs2) * inv2psi;
-    a.Tb_out[id] = a.Tb_out[id] + pb * k2 * dpt * inv2psi;
+    if (!(m & kSolid)) rp = pb * k2 * (e.dpdr - cs2) * inv2psi;
+    a.Tb_out[id] = a.Tb_out[id] + pb * k2 * e.dpdT * inv2psi;
   }
   if (m & kSolid) return;
   C fb[9];

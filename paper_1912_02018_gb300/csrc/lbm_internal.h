@@ -279,7 +279,7 @@ struct AdjArgs {
   int do_hf;
 };
 
-// One reverse step of the time step (8 launches); returns the number of launches or -1.
+// One reverse step of the time step (5 launches); returns the number of launches or -1.
 int adjoint_step_f32(const AdjArgs<float>& a, cudaStream_t s);
 int adjoint_step_f64(const AdjArgs<double>& a, cudaStream_t s);
 // Per-device set-up of the adjoint kernels (shared-memory opt-in); 0 or -1.
