@@ -159,8 +159,15 @@ __device__ __forceinline__ float theta_of(const StepConst& k, float T) {
   const float t = __fsub_rn(T, k.T_sat);
   return t == 0.0f ? 0.0f : __fsub_rn(t, k.dT_sat);
 }
+__device__ __forceinline__ float T_of(const StepConst& k, float theta) {
+  // the nearest temperature that can be stored.  The stored T_sat stands for theta = 0 and lies dT_sat off the
+  // even spacing, so its two boundaries are dT_sat / 2 off the even ones: rounded evenly there, a bulk that
+  // fluctuates about T_sat would drift by a fraction of dT_sat each step
+  const float d = fabsf(theta) < k.T_ulp ? __fmul_rn(0.5f, k.dT_sat) : k.dT_sat;
+  return __fadd_rn(k.T_sat, __fadd_rn(theta, d));
+}
 __device__ __forceinline__ float2 T_of(const StepConst& k, float2 theta) {
-  return add2(f2(k.T_sat), add2(theta, f2(k.dT_sat)));
+  return make_float2(T_of(k, theta.x), T_of(k, theta.y));
 }
 
 // Block-level end of the wall heat flux: one FP64 partial per tile column and 4-row group of the

@@ -1,0 +1,42 @@
+"""What the FP32 step rounds must not drift: errors that are the same at every node and step add up, where
+independent ones average out."""
+import numpy as np
+import pytest
+
+import synthetic_inputs as si
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+
+    from paper_1912_02018_gb300 import build
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build()
+    torch.cuda.set_device(0)
+
+
+# T_sat lies -0.48 and +0.40 of its FP32 last place off the number it is stored as
+@pytest.mark.parametrize("Tr_sat", [0.86, 0.85])
+def test_bulk_temperature_stays_at_T_sat(Tr_sat):
+    # The stored T_sat stands for T_sat itself; the bulk fluctuates about it by a few last places.  Rounding that
+    # favours one side moves its mean by a fraction of a last place every few steps (one last place in 50
+    # steps), unbiased rounding by 0.29 sqrt(60) / sqrt(nodes), far below the bar of a quarter of one.
+    from paper_1912_02018_gb300 import Sim
+
+    case = si.cylinder_case(256, 128, 16.0, Re=300.0, superheat_Tc=0.05, Tr_sat=Tr_sat, seed=3)
+    drho, theta = case.drho(), []
+    for f64 in (True, False):
+        sim = Sim.from_case(case, f64=f64, init={"drho": drho}).step(60)
+        T, T_sat = sim.fields(("T",))["T"], sim.info()["T_sat"]
+        theta.append(np.where(T == np.float32(T_sat), 0.0, T - T_sat) if not f64 else T - T_sat)
+        solid = sim.fields(("solid",))["solid"] == 1
+        sim.close()
+    ulp = float(np.spacing(np.float32(T_sat)))
+    bulk = ~solid & (np.abs(theta[0]) < 100 * ulp)
+    assert bulk.sum() > 0.5 * bulk.size
+    assert abs((theta[1] - theta[0])[bulk].mean()) < 0.25 * ulp
