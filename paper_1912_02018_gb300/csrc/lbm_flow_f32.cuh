@@ -51,15 +51,18 @@ struct PairStore<double> {
 };
 
 // Moments of a pair's pulled populations that the collision keeps: rho (in the order of pop_sum),
-// m1, m2, m4, m5 (App. A).
+// m1, m2, m4, m5 (App. A), and f_0 and the sum of the other eight.
 struct PairMoments {
-  float2 rho, m1, m2, m4, m5;
+  float2 rho, m1, m2, m4, m5, f0, sum8;
 };
 __device__ __forceinline__ PairMoments moments_pair(const float2 f[9]) {
   const float2 s12 = add2(f[1], f[2]), s34 = add2(f[3], f[4]), s56 = add2(f[5], f[6]), s78 = add2(f[7], f[8]);
   const float2 d56 = sub2(f[5], f[6]), d78 = sub2(f[7], f[8]);
   PairMoments M;
-  M.rho = add2(add2(f[0], add2(s12, s34)), add2(s56, s78));
+  const float2 s14 = add2(s12, s34), s58 = add2(s56, s78);
+  M.rho = add2(add2(f[0], s14), s58);
+  M.f0 = f[0];
+  M.sum8 = add2(s14, s58);
   M.m1 = add2(add2(sub2(f[1], f[2]), d56), d78);
   M.m2 = sub2(add2(sub2(f[3], f[4]), d56), d78);
   M.m4 = sub2(s12, s34);
@@ -87,7 +90,9 @@ __device__ __forceinline__ void force_pair(const Phys& ph, float2 rho, float2 ps
 //   k4 = m4 - u (m1 - h_x) + v (m2 - h_y),   k5 = m5 - v m1 + u h_y.
 // Raw moments from the post-collision central moments K_ab one axis at a time:
 //   M_1b = K_1b + u K_0b,  M_2b = K_2b + u (K_1b + M_1b), then the same with v over b;
-// M_10 = m1 + F_x and M_01 = m2 + F_y hold exactly.
+// M_10 = m1 + F_x and M_01 = m2 + F_y hold exactly.  f*_0 is f_0 less what the other eight gain
+// (their sum after is M_20 + M_02 - M_22): taken from the rounded rho, a quiet liquid's mass drifts by
+// up to half of rho's last place a step, the same at every node.
 // out(i, f*_i): called as each population is ready.
 template <typename Out>
 __device__ __forceinline__ void collide_pair(const StepConst& k, const PairMoments& M, float2 Fx, float2 Fy, float2 aF,
@@ -118,7 +123,7 @@ __device__ __forceinline__ void collide_pair(const StepConst& k, const PairMomen
   const float2 m21 = fma2(v, m20, M21), m22 = fma2(v, add2(M21, m21), M22);
   // f* = M^{-1} m*
   const float2 px = sub2(m20, m22), py = sub2(m02, m22);
-  out(0, sub2(sub2(rho, m20), py));
+  out(0, add2(M.f0, sub2(M.sum8, add2(m20, py))));
   const float2 hpx = mul2(f2(0.5f), px), qx = sub2(m10, m12);
   out(1, fma2(f2(0.5f), qx, hpx));
   out(2, fma2(f2(-0.5f), qx, hpx));
