@@ -151,14 +151,7 @@ __device__ __forceinline__ float lam_cv(const StepConst& k, float rho) {
   return __fmul_rn(rho, __fmaf_rn(__saturatef(__fmaf_rn(rho, k.ph1, k.ph0)), k.da, k.av));
 }
 
-// theta = T - T_sat of a stored temperature, and back.  The stored T_wall and T_sat stand for their FP64
-// values: their rounding to FP32 would reach the heat flux as a constant error (up to 1e-5 of it at a
-// superheat of 0.01 T_c).
-__device__ __forceinline__ float theta_of(const StepConst& k, float T) {
-  if (T == k.T_wall) return k.th_wall;
-  const float t = __fsub_rn(T, k.T_sat);
-  return t == 0.0f ? 0.0f : __fsub_rn(t, k.dT_sat);
-}
+// The stored temperature of theta = T - T_sat (theta_of of lbm_kernels.cuh is the way back).
 __device__ __forceinline__ float T_of(const StepConst& k, float theta) {
   // the nearest temperature that can be stored.  The stored T_sat stands for theta = 0 and lies dT_sat off the
   // even spacing, so its two boundaries are dT_sat / 2 off the even ones: rounded evenly there, a bulk that
@@ -215,7 +208,7 @@ __device__ __forceinline__ void heat_flux_groups(const Geo& g, double q, int min
 // tile also evaluates psi of the next step at its nodes from the pull of the populations this
 // step's collision wrote (fnew, side_new).
 // maps: tensor maps of the inputs, with which an interior tile stages them by TMA (else null:
-// plain loads); t1_out: where to store the stage-1 temperature (the adjoint's recompute).
+// plain loads); t1_out: where to store theta of stage 1 (the adjoint's recompute).
 template <typename S, int PSI, bool PULL, int TY>
 __device__ __forceinline__ void energy_strip(const Geo& g, const Phys& ph, const float* __restrict__ Tin,
                                              float* __restrict__ Tout, const float* __restrict__ rho,
@@ -422,7 +415,7 @@ __device__ __forceinline__ void energy_strip(const Geo& g, const Phys& ph, const
       if ((m[j] & (kSolid << 8)) && xl + 1 < g.nx) out[j].y = Tin[id + 1];
       // the row pitch is even: a pair whose right node lies past an odd nx ends in the padding
       *reinterpret_cast<float2*>(Tout + id) = out[j];
-      if (t1_out) *reinterpret_cast<float2*>(t1_out + id) = T_of(k, t1);
+      if (t1_out) *reinterpret_cast<float2*>(t1_out + id) = t1;
     }
     if (PULL && psi_out) {
       if (lane_out) {

@@ -93,7 +93,7 @@ struct Dev {
   void* T[2];        // temperature (ping-pong)
   void* psi;         // pseudopotential of the current step
   void* psi_next;    // pseudopotential of the next step, when the energy pass computed it
-  void* t1_out;      // if set, the energy pass also stores its stage-1 temperature T1 here
+  void* t1_out;      // if set, the energy pass also stores its stage-1 temperature here (FP32: T1 - T_sat)
   void* lam;         // lambda(rho) of the last collision (FP64 energy pass)
   void* en64;        // work planes of the FP64 energy pass: T1 and six frozen parts
   void* rho;         // density of the last collision
@@ -257,7 +257,7 @@ struct AdjArgs {
   const C* psi;
   const C* ux;
   const C* uy;
-  const C* T1;    // the step's stage-1 temperature (stored by its recompute)
+  const C* T1;    // the step's stage-1 temperature (stored by its recompute; in FP32 less T_sat)
   // adjoint seeds on the step's outputs, and the results on its inputs
   const C* fb_in;
   const C* Tb_in;

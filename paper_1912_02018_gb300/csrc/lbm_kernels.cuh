@@ -342,6 +342,16 @@ __device__ __forceinline__ C lam_of(const Phys& ph, C rho) {
   return mul(mul(rho, pc<C>(ph).c_v), alpha);
 }
 
+// theta = T - T_sat of a temperature stored in FP32, which the FP32 energy pass and its adjoint work with.  The
+// stored T_wall and T_sat stand for their FP64 values: their rounding to FP32 would reach the heat flux as a
+// constant error (up to 1e-5 of it at a superheat of 0.01 T_c).  Other wall temperatures, of a profile
+// along the wall or of a restored state, keep their rounding.
+__device__ __forceinline__ float theta_of(const StepConst& k, float T) {
+  if (T == k.T_wall) return k.th_wall;
+  const float t = __fsub_rn(T, k.T_sat);
+  return t == 0.0f ? 0.0f : __fsub_rn(t, k.dT_sat);
+}
+
 // ---------------------------------------------------------------- stencils on tiles (Sec. II.C)
 // p points at the stencil centre of a row-major tile with row stride s.
 // Isotropic gradient sum_k w_k phi(x+e_k) e_k over +/- pairs.
