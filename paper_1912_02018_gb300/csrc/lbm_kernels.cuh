@@ -1323,9 +1323,10 @@ static __global__ void k_export_solid(Geo g, const uint8_t* __restrict__ mask, d
 
 // Component comp (0: x, 1: y) of the force F = F_m + F_g (+ the body force) that the collision
 // applied at every node (Eq. interForce with gravity along -x, Sec. IV.A), recomputed from the
-// psi and rho that collision used with the same stencil code and roundings; zero on solid nodes
-// and when the step ran without forcing (warm-up).
-template <typename C>
+// psi and rho that collision used with the same order of operations and roundings (those of
+// force_pair and grad_rows for FP32 and FP64 populations in the FP32 build, of collide_node else); zero
+// on solid nodes and when the step ran without forcing (warm-up).
+template <typename C, typename S>
 __global__ void k_export_force(Geo g, Phys ph, const C* __restrict__ psi, const C* __restrict__ rho,
                                const uint8_t* __restrict__ mask, int forcing, int comp, double* __restrict__ dst) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1333,6 +1334,7 @@ __global__ void k_export_force(Geo g, Phys ph, const C* __restrict__ psi, const 
   if (x >= g.nx || y >= g.ny) return;
   const int id = y * g.pitch + x;
   double out = 0.0;
+  constexpr bool rows = sizeof(C) == 4 && sizeof(S) != 2;
   if (forcing && !(mask[id] & kSolid)) {
     const PhysC<C>& k = pc<C>(ph);
     const C cs2 = C(1.0 / 3.0);
@@ -1344,7 +1346,7 @@ __global__ void k_export_force(Geo g, Phys ph, const C* __restrict__ psi, const 
 #pragma unroll
         for (int c = 0; c < 5; ++c) w[r * 5 + c] = psi[map_y(g, y + r - 2) * g.pitch + map_x(g, x + c - 2)];
       C sx, sy;
-      if constexpr (sizeof(C) == 4) {
+      if constexpr (rows) {
         grad_window(w, sx, sy);
         const C a = mul(ph.sc.gm, w[12]);
         Fmx = mul(a, sx);
@@ -1356,7 +1358,7 @@ __global__ void k_export_force(Geo g, Phys ph, const C* __restrict__ psi, const 
       }
     }
     C Fx;
-    if constexpr (sizeof(C) == 4) Fx = mad(-k.g, sub(rho[id], k.rho_l), Fmx);
+    if constexpr (rows) Fx = mad(-k.g, sub(rho[id], k.rho_l), Fmx);
     else Fx = sub(Fmx, mul(sub(rho[id], k.rho_l), k.g));
     if (k.body_fx != C(0)) Fx = add(Fx, k.body_fx);
     out = comp == 0 ? (double)Fx : (double)Fmy;
@@ -1506,7 +1508,7 @@ int export_impl(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, i
   } else if (which == 5) {
     k_export_solid<<<dim3((g.nx + 255) / 256, g.ny), blk, 0, s>>>(g, d.mask, dst);
   } else if (which >= 30 && which < 34) {  // 30 + comp + 2 forcing: the force of the last collision
-    k_export_force<C><<<dim3((g.nx + 255) / 256, g.ny), blk, 0, s>>>(
+    k_export_force<C, S><<<dim3((g.nx + 255) / 256, g.ny), blk, 0, s>>>(
         g, ph, static_cast<const C*>(d.psi), static_cast<const C*>(d.rho), d.mask, (which - 30) >> 1, (which - 30) & 1,
         dst);
   } else {
