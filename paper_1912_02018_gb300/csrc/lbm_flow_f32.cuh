@@ -298,10 +298,11 @@ __device__ __forceinline__ void flow_tile(const Geo& g, const Phys& ph, const S*
     }
     M = moments_pair(fo);
     if (!landed) M.rho = f2(ph.f.rho_s);  // reported below; psi of a density that can be
-    if ((m & (kSolid * 0x0101u)) || off) {
-      if ((m & kSolid) || (off & 1u)) M.rho.x = ph.f.rho_s;
-      if ((m & (kSolid << 8)) || (off & 2u)) M.rho.y = ph.f.rho_s;
-    }
+    if (m & kSolid) M.rho.x = ph.f.rho_s;
+    if (m & (kSolid << 8)) M.rho.y = ph.f.rho_s;
+    // saturated liquid where no stencil reads: the edge column's T may have no psi at another density
+    if (off & 1u) M.rho.x = ph.f.rho_l, psi.x = ph.f.T_sat;
+    if (off & 2u) M.rho.y = ph.f.rho_l, psi.y = ph.f.T_sat;
   }
   if (multi) {
     if (MODE == kFlowTile)

@@ -63,3 +63,22 @@ def test_fp32_step_at_tile_edges(monkeypatch, nx, ny, D, periodic_x, G, storage)
             assert err <= 1e-5 * np.abs(ref.field(k)[fluid]).max(), (k, err)
     hg, hr = runs[0].heat_flux(), ref.heat_flux()
     assert hg["count"] == hr["count"] and abs(hg["q_mean"] - hr["q_mean"]) <= 1e-3 * abs(hr["q_mean"])
+
+
+@pytest.mark.parametrize("f64", [True, False])
+def test_hot_vapour_at_the_outlet_is_no_fault(f64):
+    # Vapour at 2.3 T_c in the last columns has a psi (p < rho / 3); liquid at that temperature has none.  The
+    # last tile reaches past the outlet (64 columns in tiles of 60), where nothing may be evaluated from a
+    # density that is not there.
+    from paper_1912_02018_gb300 import Sim
+
+    case = si.Case(nx=64, ny=200, D=10.0, xc=16.0, yc=100.0, Re=30.0, superheat_Tc=0.05, noise_amp=0.0)
+    probe = Sim.from_case(case, f64=True)
+    info = probe.info()
+    probe.close()
+    x = np.arange(case.nx)
+    T = info["T_sat"] + (2.3 * info["Tc"] - info["T_sat"]) * np.clip((x - 40) / 20.0, 0.0, 1.0)
+    shape = (case.ny, case.nx)
+    sim = Sim.from_case(case, f64=f64, init={"rho": np.full(shape, info["rho_v"]), "T": np.tile(T, (case.ny, 1))})
+    sim.step(2).sync()
+    sim.close()
