@@ -292,7 +292,8 @@ __device__ __forceinline__ void flow_tile(const Geo& g, const Phys& ph, const S*
       float t[9];
 #pragma unroll
       for (int q2 = 0; q2 < 9; ++q2) t[q2] = at(q2, -cxv(q2), -cyv(q2));
-      pull_special<float>(g, ph, side_in, mine ? side_out : nullptr, x, yy, (uint8_t)(m >> (8 * i)), t, at);
+      // a tile whose copy did not land stores no outlet values
+      pull_special<float>(g, ph, side_in, mine && landed ? side_out : nullptr, x, yy, (uint8_t)(m >> (8 * i)), t, at);
 #pragma unroll
       for (int q2 = 0; q2 < 9; ++q2) pair_set(fo[q2], i, t[q2]);
     }

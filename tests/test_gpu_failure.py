@@ -98,3 +98,24 @@ def test_inject_fault_rejects_an_unknown_kind():
     assert N.lib().lbm_inject_fault(sim.h, C.c_int32(7)) == N.LBM_EINVAL
     sim.step(1).sync()
     sim.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f64"])
+def test_a_starved_outlet_tile_stores_no_outlet_values(storage):
+    # The outlet rows ping-pong: the second step writes where the first step's input lies.  Staged tiles (all
+    # but the first and last rows of tiles) have nothing to write when their copies never arrive.
+    from paper_1912_02018_gb300 import Sim
+    from paper_1912_02018_gb300._native import LbmError
+
+    case = si.cylinder_case(160, 100, 16.0, Re=30.0, superheat_Tc=0.05)  # 16000 nodes, tiles of 12 or 4 rows
+    sim = Sim.from_case(case, f64=False, storage=storage)
+    first = sim.get_state_native()[2]
+    sim.step(1)
+    assert not np.array_equal(sim.get_state_native()[2], first)
+    sim.inject_fault("collide")
+    sim.step(1)
+    with pytest.raises(LbmError, match="ETIMEOUT"):
+        sim.sync()
+    sim.set_state_native()  # clears the latched fault and changes nothing
+    assert np.array_equal(sim.get_state_native()[2][:, 16:72], first[:, 16:72])
+    sim.close()
