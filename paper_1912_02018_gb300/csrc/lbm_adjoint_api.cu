@@ -38,7 +38,11 @@ struct lbm_adjoint_work {
   // ping-pong parity, heat-flux weight)
   cudaStream_t gs = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-  std::map<std::tuple<int, int, double>, cudaGraphExec_t> graphs;
+  struct Segment {
+    cudaGraphExec_t exec;
+    int launches;  // kernels in it
+  };
+  std::map<std::tuple<int, int, double>, Segment> graphs;
 };
 
 namespace {
@@ -186,15 +190,21 @@ int reverse_slot(lbm_ctx* c, lbm_adjoint_work* w, int j, int ping, double wq, cu
 }
 
 // Recompute a segment of len steps from state slot 0 and run its reverse steps, the first with
-// adjoint buffers [ping]; on stream st.  Returns false on a launch error.
-bool segment_launches(lbm_ctx* c, lbm_adjoint_work* w, int len, int ping, double wq, cudaStream_t st) {
-  for (int j = 0; j < len; ++j)
-    if (forward_slot(c, w, j, st) < 0) return false;
+// adjoint buffers [ping]; on stream st.  Returns the number of kernels launched, or -1 on a launch error.
+int segment_launches(lbm_ctx* c, lbm_adjoint_work* w, int len, int ping, double wq, cudaStream_t st) {
+  int n = 0;
+  for (int j = 0; j < len; ++j) {
+    const int k = forward_slot(c, w, j, st);
+    if (k < 0) return -1;
+    n += k;
+  }
   for (int j = len - 1; j >= 0; --j) {
-    if (reverse_slot(c, w, j, ping, wq, st) < 0) return false;
+    const int k = reverse_slot(c, w, j, ping, wq, st);
+    if (k < 0) return -1;
+    n += k;
     ping ^= 1;
   }
-  return true;
+  return n;
 }
 
 // The same from a cached CUDA graph (captured on first use).
@@ -210,20 +220,21 @@ lbm_status segment_graph(lbm_ctx* c, lbm_adjoint_work* w, int len, int ping, dou
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     LBM_CUDA(c, cudaStreamBeginCapture(w->gs, cudaStreamCaptureModeThreadLocal));
-    const bool ok = segment_launches(c, w, len, ping, wq, w->gs);
+    const int launches = segment_launches(c, w, len, ping, wq, w->gs);
     const cudaError_t e = cudaStreamEndCapture(w->gs, &graph);
-    if (!ok || e != cudaSuccess) {
+    if (launches < 0 || e != cudaSuccess) {
       if (graph) cudaGraphDestroy(graph);
       return fail(c, LBM_ECUDA, "capture of the adjoint segment failed: %s", cudaGetErrorString(cudaGetLastError()));
     }
     const cudaError_t ei = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     if (ei != cudaSuccess) return fail(c, LBM_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(ei));
-    it = w->graphs.emplace(key, exec).first;
+    it = w->graphs.emplace(key, lbm_adjoint_work::Segment{exec, launches}).first;
   }
   LBM_CUDA(c, cudaEventRecord(w->ev_in, c->stream));
   LBM_CUDA(c, cudaStreamWaitEvent(w->gs, w->ev_in, 0));
-  LBM_CUDA(c, cudaGraphLaunch(it->second, w->gs));
+  LBM_CUDA(c, cudaGraphLaunch(it->second.exec, w->gs));
+  c->launches += it->second.launches;
   LBM_CUDA(c, cudaEventRecord(w->ev_out, w->gs));
   LBM_CUDA(c, cudaStreamWaitEvent(c->stream, w->ev_out, 0));
   return LBM_OK;
@@ -352,7 +363,7 @@ namespace host {
 void adjoint_release(lbm_ctx* c) {
   if (!c->adjw) return;
   cudaStreamSynchronize(c->stream);
-  for (auto& kv : c->adjw->graphs) cudaGraphExecDestroy(kv.second);
+  for (auto& kv : c->adjw->graphs) cudaGraphExecDestroy(kv.second.exec);
   if (c->adjw->gs) {
     cudaStreamSynchronize(c->adjw->gs);
     cudaStreamDestroy(c->adjw->gs);
@@ -427,7 +438,6 @@ lbm_status lbm_adjoint_window(lbm_ctx* c, int64_t n, int32_t ckpt_every, lbm_win
     if ((st = copy_slot(c, w->sf[0], w->sT[0], w->sside[0], w->cf[s], w->cT[s], w->cside[s])) != LBM_OK) return st;
     if ((st = segment_graph(c, w, len, ping, wq)) != LBM_OK) return st;
     ping ^= len & 1;
-    c->launches += 7 * (int64_t)len + 1;
   }
   if (aux(c, 1, w->Tb[ping], w->gw) < 0) return fail(c, LBM_ECUDA, "wall seed failed");
   std::vector<double> gw;
