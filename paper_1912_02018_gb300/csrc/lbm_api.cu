@@ -1257,7 +1257,8 @@ namespace {
 
 // Tuning cache: the variant chosen for a set of domains on a kind of device, kept for the
 // process and, when the environment names a file in LBM_TUNE_CACHE, in that file (lines
-// "<16 hex digits of the key> <variant>", appended as choices are made).
+// "<16 hex digits of the key> <variant>", appended as choices are made).  The key covers the device, the
+// precision, the tiles the variants stand for and the domains.
 std::mutex g_tune_mu;
 std::map<unsigned long long, int>* g_tune = nullptr;
 
@@ -1280,6 +1281,12 @@ unsigned long long tune_key(const lbm_batch* b) {
   }
   const int f64 = b->f64 ? 1 : 0;
   h = fnv1a(h, &f64, sizeof(f64));
+  // what the variant numbers stand for: a file kept from a build with other tiles holds choices among those
+  for (int v = 0; v < lbm::kBatchVariants; ++v) {
+    int t[4] = {b->f64 ? lbm::kEnergyTX64 : lbm::kFlowTX, 0, b->f64 ? lbm::kEnergyTX64 : lbm::kEnergyTX32, 0};
+    lbm::batch_variant(v, b->f64, t[1], t[3]);
+    h = fnv1a(h, t, sizeof(t));
+  }
   for (const lbm_ctx* c : b->ctx) {
     const int dims[6] = {c->dom.nx, c->dom.ny, c->dom.periodic_x, c->dom.walls, c->prm.energy, c->prm.G != 0.0};
     const double cyl[3] = {c->cyl.D, c->cyl.xc, c->cyl.yc};
