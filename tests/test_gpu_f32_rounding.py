@@ -125,3 +125,22 @@ def test_fp32_window_gradient_is_free_of_systematic_error():
             err[k].append((out[1][k] - out[0][k]) / out[0][k])
     assert np.sqrt(np.mean(np.square(err["u_in"]))) < 80 * 0.4 * 2.0 ** -24, err
     assert np.sqrt(np.mean(np.square(err["J"]))) < 40 * 0.4 * 2.0 ** -24, err
+
+
+def test_fp32_adjoint_on_odd_sides():
+    # Window gradients on lattices whose sides are no multiples of a tile, FP32 against FP64: the FP32 bar of the
+    # adjoint tests, 1e-3
+    from paper_1912_02018_gb300 import Sim
+
+    for nx, ny, periodic_x in ((131, 97, 0), (125, 99, 1), (61, 45, 0)):
+        case = si.Case(nx=nx, ny=ny, D=14.0, xc=nx / 3.0, yc=ny / 2.0 + 0.2, Re=300.0, superheat_Tc=0.05, seed=nx,
+                       periodic_x=periodic_x, wall_dT=tuple(0.01 * si.uniform_pm1(3, 16)))
+        out = []
+        for f64 in (True, False):
+            sim = Sim.from_case(case, f64=f64, init={"drho": case.drho()}).step(20)
+            out.append(sim.adjoint_window(60, ckpt_every=25, per_node=True))
+            sim.close()
+        for k in ("J", "superheat"):
+            assert abs(out[1][k] - out[0][k]) <= 1e-3 * abs(out[0][k]), (nx, k)
+        for k in ("Tw", "wall_dT"):
+            assert np.abs(out[1][k] - out[0][k]).max() <= 1e-3 * np.abs(out[0][k]).max(), (nx, k)

@@ -82,3 +82,50 @@ def test_hot_vapour_at_the_outlet_is_no_fault(f64):
     sim = Sim.from_case(case, f64=f64, init={"rho": np.full(shape, info["rho_v"]), "T": np.tile(T, (case.ny, 1))})
     sim.step(2).sync()
     sim.close()
+
+
+@pytest.mark.parametrize("nx,ny,D,periodic_x,storage,psi_mode,collision", [
+    # psi evaluated as IEEE FP64 (by the energy pass, for the collision to read) and as FP32 (in the collision's
+    # tiles), below and above 12000 nodes and 152 energy tiles
+    (61, 33, 9.0, 0, "f32", 1, 0), (243, 61, 20.0, 1, "f32", 1, 0), (541, 245, 40.0, 0, "f32", 1, 0),
+    (600, 257, 40.0, 1, "f32", 1, 0),
+    (61, 33, 9.0, 0, "f32", 2, 0), (243, 61, 20.0, 1, "f32", 2, 0), (541, 245, 40.0, 0, "f32", 2, 0),
+    (600, 257, 40.0, 1, "f32", 2, 0),
+    # FP64 populations: psi from the energy pass's second pull, in 4- and 16-row tiles
+    (61, 33, 9.0, 1, "f64", 0, 0), (541, 245, 40.0, 0, "f64", 0, 0), (600, 257, 40.0, 1, "f64", 0, 0),
+    (541, 245, 40.0, 1, "f64", 1, 0), (243, 61, 20.0, 0, "f64", 2, 0), (600, 257, 40.0, 0, "f64", 2, 0),
+    # the BGK operator over both ways to psi
+    (61, 33, 9.0, 0, "f32", 0, 1), (243, 61, 20.0, 0, "f32", 0, 1), (243, 61, 20.0, 1, "f64", 0, 1),
+])
+def test_fp32_psi_routes_and_restart(nx, ny, D, periodic_x, storage, psi_mode, collision):
+    # against the oracle with the tolerance of the test above, and bit for bit against a run restored midway,
+    # whose first psi comes from k_rho_psi where the other run's comes from the energy pass or the tile
+    from paper_1912_02018_gb300 import Sim
+
+    case = si.Case(nx=nx, ny=ny, D=D, xc=nx / 3.0 - 0.3, yc=ny / 2.0 + 0.2, Re=40.0, superheat_Tc=0.08, nu_ratio=1.5,
+                   periodic_x=periodic_x, seed=nx + psi_mode, collision=collision)
+    drho = case.drho()
+    kw = dict(f64=False, storage=storage, psi_mode=psi_mode)
+    sim = Sim.from_case(case, init={"drho": drho}, **kw).step(5)
+    state = sim.get_state_native()
+    sim.step(5)
+    again = Sim.from_case(case, **kw)
+    again.set_state_native(*state)
+    again.step(5)
+    names = ("rho", "ux", "uy", "T", "psi", "Fx", "Fy")
+    got, restored = sim.fields(names), again.fields(names)
+    for k in names:
+        assert np.array_equal(got[k], restored[k]), k
+    for a, b in zip(sim.get_state_native(), again.get_state_native()):
+        assert np.array_equal(a, b)
+    ref = Oracle(case, drho=drho).step(10)
+    fluid = ref.field("solid") == 0
+    speed = np.hypot(ref.field("ux"), ref.field("uy"))[fluid].max()
+    for k in ("rho", "ux", "uy", "T", "psi"):
+        err = np.abs(got[k] - ref.field(k))[fluid].max()
+        if k in ("ux", "uy"):
+            assert err <= 1e-3 * speed, (k, err)
+        else:
+            assert err <= 1e-5 * np.abs(ref.field(k)[fluid]).max(), (k, err)
+    sim.close()
+    again.close()
