@@ -88,7 +88,7 @@ lbm_status prepare(lbm_ctx* c, int K, int nseg) {
     w->auy.push_back(ruv ? ruv + 2 * plane : nullptr);
     w->aT1.push_back(A(plane));
   }
-  for (int j = 0; j <= K; ++j) w->apsi.push_back(A(plane));  // psi of slot K comes from the last energy pass
+  for (int j = 0; j <= K; ++j) w->apsi.push_back(A(plane));  // FP64: slot K takes psi of the last energy pass
   for (int s = 0; s < nseg; ++s) {
     w->cf.push_back(A(fs));
     w->cT.push_back(A(plane));
@@ -118,9 +118,9 @@ lbm_status prepare(lbm_ctx* c, int K, int nseg) {
   return LBM_OK;
 }
 
-// Forward step of slot j into slot j + 1, keeping the collision fields of slot j.  Within a
-// segment the energy pass of step j makes psi of step j + 1, so only the first step runs the psi
-// pass.
+// Forward step of slot j into slot j + 1, keeping the collision fields of slot j.  Within a segment psi of
+// step j + 1 comes from the energy pass of step j (FP64) or the collision of step j + 1 (FP32), so at most
+// the first step runs a psi pass.
 int forward_slot(lbm_ctx* c, lbm_adjoint_work* w, int j, cudaStream_t st) {
   lbm::Dev v = c->dev;
   v.f[0] = w->sf[j];
@@ -141,7 +141,7 @@ int forward_slot(lbm_ctx* c, lbm_adjoint_work* w, int j, cudaStream_t st) {
   // passes (512 x 256: one wave each) measured slower there
   v.pdl = 0;
   int flipped = 0;
-  lbm::PsiChain chain{j > 0 ? 1 : 0, 1, 0};
+  lbm::PsiChain chain{j == 0 ? lbm::kPsiFromPass : lbm::kPsiFromPlane, 1, 0};  // (kPsiFromTile does the same)
   const int k = c->f64 ? lbm::step_f64(c->geo, c->ph, v, 0, 0, 1, 1, c->prm.psi_mode, st, nullptr, &flipped, &chain)
                        : lbm::step_f32(c->geo, c->ph, v, 0, 0, 1, 1, c->prm.psi_mode, c->prm.storage, st, nullptr,
                                        &flipped, &chain);

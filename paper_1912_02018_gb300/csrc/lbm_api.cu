@@ -717,7 +717,7 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
     const int forcing = c->steps >= c->prm.warmup_steps;
     int flipped = 0;
     // psi of this step may already have been made by the last energy pass (into psi_next)
-    if (c->psi_pending) std::swap(c->dev.psi, c->dev.psi_next);
+    if (c->psi_pending == lbm::kPsiFromPlane) std::swap(c->dev.psi, c->dev.psi_next);
     lbm::PsiChain chain{c->psi_pending, 1, 0};
     // from the second step of a call on, the kernel before the collision is the last step's
     // energy pass, which leaves the populations alone
@@ -1048,7 +1048,7 @@ static lbm_status batch_layout(lbm_batch* b) {
     const int ntx = (g.nx + 31) / 32;
     D.psi_first = (int)mp.size();
     D.psi_ntx = ntx;
-    mp.insert(mp.end(), (size_t)ntx * ((g.ny + 7) / 8), (int)k);
+    if (b->f64) mp.insert(mp.end(), (size_t)ntx * ((g.ny + 7) / 8), (int)k);
     D.coll_first = (int)mc.size();
     D.coll_ntx = b->f64 ? ntx : (g.nx + lbm::kFlowTX - 1) / lbm::kFlowTX;
     mc.insert(mc.end(), (size_t)D.coll_ntx * ((g.ny + cty - 1) / cty), (int)k);
@@ -1068,7 +1068,7 @@ static lbm_status batch_layout(lbm_batch* b) {
     return batch_fail(b, LBM_ESTATE, "batch tile maps larger than allocated");
   cudaError_t e = cudaMemcpyAsync(b->d_doms, b->h_doms.data(), sizeof(lbm::BatchDomain) * b->h_doms.size(),
                                   cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !mp.empty())
     e = cudaMemcpyAsync(b->d_maps, mp.data(), sizeof(int) * mp.size(), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->d_maps + b->max_tiles, mc.data(), sizeof(int) * mc.size(), cudaMemcpyHostToDevice,
@@ -1082,7 +1082,8 @@ static lbm_status batch_layout(lbm_batch* b) {
 }
 
 // psi of the current state is unknown for some two-phase domain (creation, or a state set
-// through the API): the next step starts with the psi pass
+// through the API): the next step starts with the psi pass in FP64.  In FP32 there is none; that step is
+// merely not replayed from a graph.
 static bool batch_needs_psi(const lbm_batch* b) {
   for (const lbm_ctx* c : b->ctx)
     if (!c->psi_pending && c->ph.d.G != 0.0) return true;
@@ -1101,10 +1102,9 @@ static int batch_launch(lbm_batch* b, cudaStream_t s) {
                                       b->h_doms.data(), b->hmaps.data(), nd, s);
 }
 
-// After a batched step: the energy pass has made psi of the new state in buffer b->cur (FP64; the
-// FP32 collision makes psi itself); each
-// domain's context sees the buffers as a single-domain step leaves them (psi: the one the
-// step's collision used, psi_next: the pending one)
+// After a batched step: each domain's context sees the buffers as a single-domain step leaves them.  psi
+// is the one that the step's collision used; psi_next is in FP64 the one of the new state, which the
+// energy pass has made in buffer b->cur, and in FP32, where the collision evaluates psi, of no use.
 static void batch_advance(lbm_batch* b, int launches) {
   b->cur ^= 1;
   b->tcur ^= 1;
@@ -1117,7 +1117,7 @@ static void batch_advance(lbm_batch* b, int launches) {
     c->launches += launches;
     c->dev.psi = b->psi_buf[b->cur ^ 1][k];
     c->dev.psi_next = b->psi_buf[b->cur][k];
-    c->psi_pending = 1;
+    c->psi_pending = b->f64 ? lbm::kPsiFromPlane : lbm::kPsiFromTile;
   }
 }
 

@@ -368,10 +368,7 @@ __device__ __forceinline__ void energy_strip(const Geo& g, const Phys& ph, const
     for (int j = 0; j < 2; ++j) {
       const float2 t = aT[j * A2 + 1];
       float2 t1 = add2(t, L[j]);
-      if (!g.periodic_x) {
-        if (xl == 0) t1.x = 0.0f;  // the inlet column stays at T_sat
-        if (xl + 1 == 0) t1.y = 0.0f;
-      }
+      if (!g.periodic_x && xl == 0) t1.x = 0.0f;  // the inlet column stays at T_sat (xl is even)
       if (m[j] & kSolid) t1.x = t.x;  // solid nodes keep their wall temperature
       if (m[j] & (kSolid << 8)) t1.y = t.y;
       bT[j * B2] = t1;  // positions past a non-periodic edge are replaced below

@@ -30,8 +30,8 @@ int batch_step_f64(int variant, const BatchDomain* doms, const int* mp, int np, 
                    const int* me, int ne, int cur, int tcur, long long step, int need_psi,
                    const BatchDomain* hd, const DomainMaps* hm, int nd, cudaStream_t s) {
   switch (variant & 1) {
-    case 1: return kern::batch_step_impl<double, double, kPsiF64, 16, 8>(doms, mp, np, mc, nc, me, ne, cur, tcur, step, need_psi, hd, hm, nd, s);
-    default: return kern::batch_step_impl<double, double, kPsiF64, 8, 8>(doms, mp, np, mc, nc, me, ne, cur, tcur, step, need_psi, hd, hm, nd, s);
+    case 1: return kern::batch_step_impl<double, double, kPsiF64, 16>(doms, mp, np, mc, nc, me, ne, cur, tcur, step, need_psi, hd, hm, nd, s);
+    default: return kern::batch_step_impl<double, double, kPsiF64, 8>(doms, mp, np, mc, nc, me, ne, cur, tcur, step, need_psi, hd, hm, nd, s);
   }
 }
 

@@ -149,8 +149,11 @@ struct DomainMaps {
   EnergyMaps em[2];
 };
 constexpr int kBatchCollDomains = 126, kBatchEnDomains = 126;
-struct CollLaunchMaps {
+struct CollLaunchMaps {  // FP64
   CUtensorMap f[kBatchCollDomains], psi[kBatchCollDomains];
+};
+struct FlowLaunchMaps {  // FP32: psi is evaluated in the tiles
+  CUtensorMap f[kBatchCollDomains];
 };
 struct EnLaunchMaps {
   EnergyMaps e[kBatchEnDomains];
@@ -204,9 +207,11 @@ struct LaunchHook {
   void* self;
 };
 
-// psi of the next step: have = this step needs no psi pass (d.psi holds its psi, or the collision
-// makes it), want = the energy pass should see to that for the next step (by writing d.psi_next,
-// where the collision does not make psi); made is set when it did.
+// Where psi of the next step comes from: a psi pass, plane psi_next (the energy pass has written it), or
+// the tiles of the next collision, which evaluate it.
+enum PsiSource { kPsiFromPass = 0, kPsiFromPlane = 1, kPsiFromTile = 2 };
+// have: the PsiSource of this step (kPsiFromPlane: already moved to d.psi); want: whether the step should
+// spare the next one its psi pass; made: the PsiSource of the next step, set by the step.
 struct PsiChain {
   int have, want, made;
 };

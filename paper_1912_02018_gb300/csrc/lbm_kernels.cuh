@@ -314,16 +314,6 @@ __device__ __forceinline__ C psi_of(const Phys& ph, C rho, C T, int* status) {
     return (C)p;
   }
 }
-// (dp/dT) at fixed rho, the derivative of Eq. (eos).
-template <typename C>
-__device__ __forceinline__ C dpdT_eos(const Phys& ph, C rho, C T) {
-  C s = C(1) + pc<C>(ph).kappa * (C(1) - sqrt(fdiv(T, pc<C>(ph).Tc)));
-  C dphi = fdiv(-pc<C>(ph).kappa * s, sqrt(T * pc<C>(ph).Tc));
-  C rep = fdiv(rho * pc<C>(ph).R, C(1) - pc<C>(ph).b * rho);
-  C att = fdiv(pc<C>(ph).a * dphi * rho * rho,
-               C(1) + C(2) * pc<C>(ph).b * rho - pc<C>(ph).b * pc<C>(ph).b * rho * rho);
-  return rep - att;
-}
 // Phase fraction for the transport properties, and nu(rho), lambda(rho).
 template <typename C>
 __device__ __forceinline__ C phase_frac(const Phys& ph, C rho) {
@@ -1186,7 +1176,7 @@ static __global__ void __launch_bounds__(128)
                static_cast<const double*>(D.d.ux), static_cast<const double*>(D.d.uy), D.d.mask, bx, by, fnew, side_new,
                psi_next, D.d.status);
 }
-template <typename C, typename S, int PSI, int CTY, int ETY>
+template <typename C, typename S, int PSI, int CTY>
 int batch_step_impl(const BatchDomain* doms, const int* map_psi, int nb_psi, const int* map_coll, int nb_coll,
                     const int* map_en, int nb_en, int cur, int tcur, long long step, int need_psi,
                     const BatchDomain* hdoms, const DomainMaps* hmaps, int ndom, cudaStream_t s) {
@@ -1488,9 +1478,9 @@ int step_impl(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int
     }
     post(kKEnergy);
     *t_flipped = 1;
-    if (chain) chain->made = fuse ? 1 : 0;
+    if (chain) chain->made = fuse ? kPsiFromPlane : kPsiFromPass;
   } else if (chain) {
-    chain->made = 0;
+    chain->made = kPsiFromPass;
   }
   return cudaPeekAtLastError() == cudaSuccess ? n : -1;
 }

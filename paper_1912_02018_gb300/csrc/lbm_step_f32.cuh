@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(EnergyTile<TY>::NT, TY == kEnergyTY ? 3 : 4)
 template <int CTY>
 __global__ void __launch_bounds__(FlowTile<float, kFlowTile, CTY>::NT, CTY == kFlowTY ? 2 : 3)
     kb_collide_f32(const BatchDomain* __restrict__ doms, const int* __restrict__ map, int cur, int tcur, long long step,
-                   int block0, int dom0, const __grid_constant__ CollLaunchMaps maps) {
+                   int block0, int dom0, const __grid_constant__ FlowLaunchMaps maps) {
   const int blk = block0 + blockIdx.x, k = map[blk];
   const BatchDomain& D = doms[k];
   const int local = blk - D.coll_first;
@@ -115,7 +115,7 @@ int batch_step_impl_f32(const BatchDomain* doms, const int* map_coll, int nb_col
   int n = 0;
   for (int d0 = 0; d0 < ndom; d0 += kBatchCollDomains) {
     const int d1 = d0 + kBatchCollDomains < ndom ? d0 + kBatchCollDomains : ndom;
-    CollLaunchMaps m;
+    FlowLaunchMaps m;
     for (int k = d0; k < d1; ++k) m.f[k - d0] = hmaps[k].f[cur];
     const int b0 = hdoms[d0].coll_first, b1 = d1 < ndom ? hdoms[d1].coll_first : nb_coll;
     kb_collide_f32<CTY><<<b1 - b0, FlowTile<float, kFlowTile, CTY>::NT, 0, s>>>(doms, map_coll, cur, tcur, step, b0, d0, m);
@@ -180,8 +180,8 @@ void launch_energy_f32(const Geo& g, const Phys& ph, const Dev& d, int cur, int 
 // A step takes the collision with psi in its tiles (populations stored in FP32, psi in FP32 or
 // double-float) or reads psi, which the energy pass of the step before has made (FP64 populations or
 // FP64 psi: their tiles would not fit shared memory, or cost more than the second pull) or, in a
-// first step, k_rho_psi.  On small lattices a first step (chain->have unset) runs k_rho_psi too, so
-// that its launches are those of every two-phase run.
+// first step, k_rho_psi.  On small lattices (flow_psi_in_tile) a step whose predecessor ran no energy pass
+// (a first step, a warm-up step, T fixed) takes psi from k_rho_psi too.
 template <typename S, int PSI>
 int step_impl_f32(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int forcing, int energy,
                   cudaStream_t s, const LaunchHook* hook, int* t_flipped, PsiChain* chain) {
@@ -212,7 +212,7 @@ int step_impl_f32(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur,
   else if constexpr (can_tile) launch_flow_f32<S, PSI, kFlowTile>(g, ph, d, cur, tcur, forcing, s);
   post(kKCollide);
   *t_flipped = 0;
-  if (chain) chain->made = 0;
+  if (chain) chain->made = kPsiFromPass;
   if (energy && forcing) {
     const bool next = chain && chain->want && multi, small = small_lattice(g.nx, g.ny);
     pre(kKEnergy);
@@ -227,7 +227,7 @@ int step_impl_f32(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur,
     }
     post(kKEnergy);
     *t_flipped = 1;
-    if (chain) chain->made = next && (!can_tile || !flow_psi_in_tile(g.nx, g.ny)) ? 1 : 0;
+    if (chain) chain->made = !next ? kPsiFromPass : can_tile ? kPsiFromTile : kPsiFromPlane;
   }
   return cudaPeekAtLastError() == cudaSuccess ? n : -1;
 }

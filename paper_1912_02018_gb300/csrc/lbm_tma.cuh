@@ -7,7 +7,8 @@
 // Copy rules kept by every caller: the tile's first column times the element size is a
 // multiple of 16 bytes, the box's inner extent is a multiple of 16 bytes, base addresses are
 // 16-byte aligned and row/plane strides multiples of 16 bytes; coordinates past the lattice
-// are read as zeros (callers use TMA only where the box lies inside the lattice).
+// are read as zeros.  Callers use TMA where the box lies inside the lattice, and in the FP32 step also at
+// an inlet or outlet, whose tiles replace what lies past the edge column.
 #pragma once
 
 #include <cuda.h>
