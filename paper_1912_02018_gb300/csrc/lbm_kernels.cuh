@@ -829,7 +829,9 @@ __device__ __forceinline__ void psi_tile_plain(const Geo& g, const C* __restrict
 }
 
 // Collision tile (bx, by) of 32 x CTY nodes.  tm_f, tm_psi: tensor maps of f and psi for TMA
-// staging, or null.
+// staging, or null.  FP64 blocks leave the next pass to start when they end: they run for 15 us on the FP64
+// pipe, and blocks of the next pass that wait beside them from the start pile up on some SMs (241 x 241,
+// single phase: 51 us a step so, 36 us now; 512 x 256: the same).
 template <typename C, typename S, int CTY, int OP = kCollCM>
 __device__ __forceinline__ void collide_tile(const Geo& g, const Phys& ph, const S* __restrict__ f,
                                              S* __restrict__ fn, const C* __restrict__ psi,
@@ -858,14 +860,14 @@ __device__ __forceinline__ void collide_tile(const Geo& g, const Phys& ph, const
       if (!starve && early_f) tma::load_3d(s_f, tm_f, &s_bar, x0 - CS::XA, y0 - 1, 0);
     }
     pdl::wait();  // psi is the previous kernel's output
-    pdl::trigger();
+    if (sizeof(C) == 4) pdl::trigger();
     if (tid == 0 && !starve) {
       if (!early_f) tma::load_3d(s_f, tm_f, &s_bar, x0 - CS::XA, y0 - 1, 0);
       if (need_psi) tma::load_2d(s_psi, tm_psi, &s_bar, x0 - CS::PA, y0 - 2);
     }
   } else {
     pdl::wait();
-    pdl::trigger();
+    if (sizeof(C) == 4) pdl::trigger();
     if (need_psi) {
       psi_tile_plain<C, S, CTY>(g, psi, x0, y0, s_psi);
       __syncthreads();
