@@ -431,17 +431,17 @@ __device__ __forceinline__ void grad_rows(const float2* q, int ts, float2& gx, f
             fma2(f2(wrow(1, 1)), sub2(hi.S1, lo.S1), fma2(f2(wrow(1, 2)), sub2(hi.S2, lo.S2), gy)));
   row_gx(row_sums<true, false>(q), 0, gx);
 }
-__device__ __forceinline__ void grad_window(const float* w, float& gx, float& gy) {
+__device__ __forceinline__ void grad_window(const float* w, int s, float& gx, float& gy) {
   gx = gy = 0.0f;
 #pragma unroll
   for (int k = 2; k >= 0; --k) {
 #pragma unroll
     for (int t = 0; t < (k ? 2 : 1); ++t) {
-      const float* q = w + 5 * (t ? 2 + k : 2 - k);
+      const float* q = w + s * (t ? 2 + k : 2 - k);
       gx = __fmaf_rn(wrow(k, 1), __fsub_rn(q[3], q[1]), __fmaf_rn(2.0f * wrow(k, 2), __fsub_rn(q[4], q[0]), gx));
     }
     if (k == 0) continue;
-    const float *a = w + 5 * (2 - k), *b = w + 5 * (2 + k);
+    const float *a = w + s * (2 - k), *b = w + s * (2 + k);
     gy = __fmaf_rn(k * wrow(k, 0), __fsub_rn(b[2], a[2]),
                    __fmaf_rn(k * wrow(k, 1), __fsub_rn(__fadd_rn(b[3], b[1]), __fadd_rn(a[3], a[1])),
                              __fmaf_rn(k * wrow(k, 2), __fsub_rn(__fadd_rn(b[4], b[0]), __fadd_rn(a[4], a[0])), gy)));
@@ -583,6 +583,12 @@ __device__ __forceinline__ C psi_node(const Geo& g, const Phys& ph, const S* __r
   }
   return psi_of<C, PSI>(ph, rho, t, status);
 }
+
+}  // namespace kern
+}  // namespace lbm
+#include "lbm_collide_f32.cuh"
+namespace lbm {
+namespace kern {
 
 // ---------------------------------------------------------------- CM collision (Sec. II.A-B)
 // Raw moments -> central moments k4, k5 (T = N M), post-collision CMs of Eq. (postColl2),
@@ -751,6 +757,8 @@ __device__ __forceinline__ bool coll_staged(const Geo& g, int x0, int y0) {
 // substitutions), interaction force from the psi tile s_psi with its 2-node halo, gravity,
 // CM collision (or, with OP = kCollBGK, the BGK comparison operator); writes f* (other
 // buffer), rho, u and the outlet's streamed values.
+// FP32 arithmetic over FP32 or FP64 populations takes the operations of lbm_collide_f32.cuh, with the bits of the
+// column pairs of lbm_flow_f32.cuh.
 template <typename C, typename S, int CTY, int OP = kCollCM>
 __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const S* __restrict__ f,
                                              S* __restrict__ fn, const C* __restrict__ psi,
@@ -767,7 +775,7 @@ __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const
     rho_o[id] = k.rho_s;
     ux_o[id] = C(0);
     uy_o[id] = C(0);
-    if (lam_o) lam_o[id] = lam_of(ph, k.rho_s);
+    if (sizeof(C) == 8 && lam_o) lam_o[id] = lam_of(ph, k.rho_s);
     return;
   }
   const bool multiphase = k.G != C(0);
@@ -786,12 +794,33 @@ __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const
   } else {
     pull_node<C, S>(g, ph, f, mask, side_in, side_out, x, y, m, fo);
   }
+  const int pc0 = (ty + 2) * HX + tx + CS::PA;  // this node in the psi tile
+  if constexpr (sizeof(C) == 4 && sizeof(S) != 2) {
+    const Moments<float> M = moments_of(fo);
+    float Fx = 0.0f, Fy = 0.0f, aF = 0.0f, ux, uy;
+    if (forcing) {
+      float gx = 0.0f, gy = 0.0f, psi0 = 0.0f;
+      if (multiphase) {
+        psi0 = s_psi[pc0];
+        grad_window(&s_psi[pc0] - 2 * HX - 2, HX, gx, gy);
+        aF = mul2(ph.sc.sg, fma2(gx, gx, mul2(gy, gy)));
+      }
+      force_of(ph, M.rho, psi0, gx, gy, Fx, Fy);
+    }
+    auto out = [&](int i, float v) { fn[i * g.plane + id] = PopIO<C, S>::st(v, i, ph); };
+    if constexpr (OP == kCollBGK) collide_bgk_of(ph.sc, fo, M, Fx, Fy, ux, uy, out);
+    else collide_cm(ph.sc, M, Fx, Fy, aF, ux, uy, out);
+    rho_o[id] = M.rho;
+    ux_o[id] = ux;
+    uy_o[id] = uy;
+    if (!(M.rho > 0.0f) || !(ux == ux) || !(uy == uy)) atomicOr(status, 1);
+    return;
+  }
   C rho = fo[0];
 #pragma unroll
   for (int i = 1; i < 9; ++i) rho = rho + fo[i];
   const C cs2 = C(1.0 / 3.0);
   C Fmx = C(0), Fmy = C(0), Fx = C(0), Fy = C(0), psi0 = C(0);
-  const int pc0 = (ty + 2) * HX + tx + CS::PA;  // this node in the psi tile
   if (multiphase) psi0 = need_psi ? s_psi[pc0] : psi[id];
   if (need_psi) {
     C sx, sy;
@@ -814,7 +843,7 @@ __device__ __forceinline__ void collide_node(const Geo& g, const Phys& ph, const
   rho_o[id] = rho;
   ux_o[id] = ux;
   uy_o[id] = uy;
-  if (lam_o) lam_o[id] = lam_of(ph, rho);
+  if (sizeof(C) == 8 && lam_o) lam_o[id] = lam_of(ph, rho);
   if (!(rho > C(0)) || !(ux == ux) || !(uy == uy)) atomicOr(status, 1);
 }
 
@@ -889,8 +918,9 @@ __device__ __forceinline__ void collide_tile(const Geo& g, const Phys& ph, const
 }
 
 template <typename C, typename S, int OP = kCollCM>
-// FP16 storage: at most 36 registers, so 7 blocks share an SM and more pulls are in flight (7 blocks
-// and a few spilled registers beat 6 without spills, 30.8 vs 32.6 us at 1536 x 768)
+// FP32 arithmetic: at most 36 registers, so 7 blocks share an SM and more pulls are in flight (7 blocks
+// and a few spilled registers beat 6 without spills: FP16 storage 30.8 vs 32.6 us at 1536 x 768, FP32 30.4 vs
+// 32.8 us at 2048 x 1024)
 __global__ void __launch_bounds__(kCollTX* kCollTY, sizeof(C) == 4 ? 7 : 1)
     k_collide(Geo g, Phys ph, const S* __restrict__ f, S* __restrict__ fn, const C* __restrict__ psi,
               const uint8_t* __restrict__ mask, const C* __restrict__ side_in, C* __restrict__ side_out,
@@ -1315,10 +1345,10 @@ static __global__ void k_export_solid(Geo g, const uint8_t* __restrict__ mask, d
 
 // Component comp (0: x, 1: y) of the force F = F_m + F_g (+ the body force) that the collision
 // applied at every node (Eq. interForce with gravity along -x, Sec. IV.A), recomputed from the
-// psi and rho that collision used with the same order of operations and roundings (those of
-// force_pair and grad_rows for FP32 and FP64 populations in the FP32 build, of collide_node else); zero
-// on solid nodes and when the step ran without forcing (warm-up).
-template <typename C, typename S>
+// psi and rho that collision used with the same order of operations and roundings (rows: those of
+// force_of and grad_rows, which the FP32 build takes but for FP16 populations; else of collide_node); zero on
+// solid nodes and when the step ran without forcing (warm-up).
+template <typename C, bool rows>
 __global__ void k_export_force(Geo g, Phys ph, const C* __restrict__ psi, const C* __restrict__ rho,
                                const uint8_t* __restrict__ mask, int forcing, int comp, double* __restrict__ dst) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1326,7 +1356,6 @@ __global__ void k_export_force(Geo g, Phys ph, const C* __restrict__ psi, const 
   if (x >= g.nx || y >= g.ny) return;
   const int id = y * g.pitch + x;
   double out = 0.0;
-  constexpr bool rows = sizeof(C) == 4 && sizeof(S) != 2;
   if (forcing && !(mask[id] & kSolid)) {
     const PhysC<C>& k = pc<C>(ph);
     const C cs2 = C(1.0 / 3.0);
@@ -1339,7 +1368,7 @@ __global__ void k_export_force(Geo g, Phys ph, const C* __restrict__ psi, const 
         for (int c = 0; c < 5; ++c) w[r * 5 + c] = psi[map_y(g, y + r - 2) * g.pitch + map_x(g, x + c - 2)];
       C sx, sy;
       if constexpr (rows) {
-        grad_window(w, sx, sy);
+        grad_window(w, 5, sx, sy);
         const C a = mul(ph.sc.gm, w[12]);
         Fmx = mul(a, sx);
         Fmy = mul(a, sy);
@@ -1403,6 +1432,31 @@ cudaError_t launch_dep(bool pdl, dim3 grd, dim3 blk, size_t smem, cudaStream_t s
   return cudaLaunchKernelEx(&cfg, k, static_cast<Args&&>(args)...);
 }
 
+// The collision of 32 x 8 tiles, one node per lane, with psi read from memory.
+template <typename C, typename S>
+void launch_collide(const Geo& g, const Phys& ph, const Dev& d, int cur, int forcing, C* lam, cudaStream_t s) {
+  using namespace kern;
+  const S* f = static_cast<const S*>(d.f[cur]);
+  const C* psi = static_cast<const C*>(d.psi);
+  // tensor maps of this step's populations and psi for the TMA-staged tiles (plain loads
+  // everywhere when a map cannot be made)
+  using CS = CollStage<C, S, kCollTY>;
+  CUtensorMap tm_f = {}, tm_psi = {};
+  const bool staged = d.tma && tma::encode<S>(&tm_f, f, g.nx, g.ny, g.pitch, g.plane, 9, CS::FW, CS::FH) &&
+                      (ph.d.G == 0.0 || tma::encode<C>(&tm_psi, psi, g.nx, g.ny, g.pitch, g.plane, 1, CS::PW, CS::PH));
+  const int flags = staged ? (kLaunchStaged | ((d.starve & kStarveCollide) ? kLaunchStarve : 0) |
+                              ((d.pdl && d.f_ready) ? kLaunchEarlyF : 0))
+                           : 0;
+  const dim3 blk(kCollTX, kCollTY), grd((g.nx + kCollTX - 1) / kCollTX, (g.ny + kCollTY - 1) / kCollTY);
+  auto go = [&](auto kernel) {
+    launch_dep(d.pdl, grd, blk, 0, s, kernel, g, ph, f, static_cast<S*>(d.f[cur ^ 1]), psi, d.mask,
+               static_cast<const C*>(d.side[cur]), static_cast<C*>(d.side[cur ^ 1]), static_cast<C*>(d.rho),
+               static_cast<C*>(d.ux), static_cast<C*>(d.uy), forcing, d.status, tm_f, tm_psi, flags, lam);
+  };
+  if (d.collision == kCollBGK) go(k_collide<C, S, kCollBGK>);
+  else go(k_collide<C, S, kCollCM>);
+}
+
 template <typename C, typename S, int PSI>
 int step_impl(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int forcing, int energy, cudaStream_t s,
               const LaunchHook* hook, int* t_flipped, PsiChain* chain) {
@@ -1431,23 +1485,9 @@ int step_impl(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int
     k_rho_psi<C, S, PSI><<<grd, blk, 0, s>>>(g, ph, f, T, d.mask, side_in, psi, d.status);
     post(kKRhoPsi);
   }
-  // tensor maps of this step's populations and psi for the TMA-staged tiles (plain loads
-  // everywhere when a map cannot be made)
-  using CS = CollStage<C, S, kCollTY>;
-  CUtensorMap tm_f, tm_psi;
-  const bool staged = d.tma && tma::encode<S>(&tm_f, f, g.nx, g.ny, g.pitch, g.plane, 9, CS::FW, CS::FH) &&
-                      tma::encode<C>(&tm_psi, psi, g.nx, g.ny, g.pitch, g.plane, 1, CS::PW, CS::PH);
   pre(kKCollide);
-  const int cflags = staged ? (kLaunchStaged | ((d.starve & kStarveCollide) ? kLaunchStarve : 0) |
-                               ((d.pdl && d.f_ready) ? kLaunchEarlyF : 0))
-                            : 0;
   C* const lam = sizeof(C) == 8 && energy && forcing ? static_cast<C*>(d.lam) : nullptr;
-  if (d.collision == kCollBGK)
-    launch_dep(d.pdl, grd, blk, 0, s, k_collide<C, S, kCollBGK>, g, ph, f, fn, psi, d.mask, side_in, side_out, rho, ux,
-               uy, forcing, d.status, tm_f, tm_psi, cflags, lam);
-  else
-    launch_dep(d.pdl, grd, blk, 0, s, k_collide<C, S, kCollCM>, g, ph, f, fn, psi, d.mask, side_in, side_out, rho, ux, uy,
-               forcing, d.status, tm_f, tm_psi, cflags, lam);
+  launch_collide<C, S>(g, ph, d, cur, forcing, lam, s);
   post(kKCollide);
   *t_flipped = 0;
   if (energy && forcing) {
@@ -1500,7 +1540,7 @@ int export_impl(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, i
   } else if (which == 5) {
     k_export_solid<<<dim3((g.nx + 255) / 256, g.ny), blk, 0, s>>>(g, d.mask, dst);
   } else if (which >= 30 && which < 34) {  // 30 + comp + 2 forcing: the force of the last collision
-    k_export_force<C, S><<<dim3((g.nx + 255) / 256, g.ny), blk, 0, s>>>(
+    k_export_force<C, (sizeof(C) == 4 && sizeof(S) != 2)><<<dim3((g.nx + 255) / 256, g.ny), blk, 0, s>>>(
         g, ph, static_cast<const C*>(d.psi), static_cast<const C*>(d.rho), d.mask, (which - 30) >> 1, (which - 30) & 1,
         dst);
   } else {

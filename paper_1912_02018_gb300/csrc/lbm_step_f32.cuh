@@ -21,20 +21,13 @@ struct EnergyTile {
 namespace lbm {
 namespace kern {
 
-// Rows of a flow tile, and blocks per SM.
-template <typename S, int MODE>
-struct FlowRows {
-  static constexpr int v = MODE == kFlowNone ? (sizeof(S) == 8 ? 6 : 8) : MODE == kFlowRead ? 4 : kFlowTY;
-  static constexpr int blocks = MODE == kFlowNone ? 4 : MODE == kFlowRead ? 4 : 2;
-};
-
-template <typename S, int PSI, int MODE, int OP>
-__global__ void __launch_bounds__(FlowTile<S, MODE, FlowRows<S, MODE>::v>::NT, FlowRows<S, MODE>::blocks)
-    k_collide_f32(Geo g, Phys ph, const S* __restrict__ f, S* __restrict__ fn, const float* __restrict__ T, float* psi,
+template <int PSI, int OP>
+__global__ void __launch_bounds__(FlowTile<kFlowTY>::NT, 2)
+    k_collide_f32(Geo g, Phys ph, const float* __restrict__ f, float* __restrict__ fn, const float* __restrict__ T, float* psi,
                   const uint8_t* __restrict__ mask, const float* __restrict__ side_in, float* __restrict__ side_out,
                   float* __restrict__ rho_o, float* __restrict__ ux_o, float* __restrict__ uy_o, int forcing,
                   int* status, const __grid_constant__ CUtensorMap tm_f, int flags) {
-  flow_tile<S, PSI, MODE, OP, FlowRows<S, MODE>::v>(g, ph, f, fn, T, psi, mask, side_in, side_out, rho_o, ux_o, uy_o,
+  flow_tile<PSI, OP, kFlowTY>(g, ph, f, fn, T, psi, mask, side_in, side_out, rho_o, ux_o, uy_o,
                                                     forcing, status, blockIdx.x, blockIdx.y,
                                                     (flags & kLaunchStaged) ? &tm_f : nullptr,
                                                     (flags & kLaunchStarve) != 0, (flags & kLaunchEarlyF) != 0);
@@ -56,13 +49,13 @@ __global__ void __launch_bounds__(EnergyTile<TY>::NT, TY == kEnergyTY ? 3 : 4)
 // A batched launch covers the blocks [block0, block0 + gridDim.x) of a pass, which belong to the
 // domains dom0 ..; their tensor maps come as kernel parameters (index k - dom0).
 template <int CTY>
-__global__ void __launch_bounds__(FlowTile<float, kFlowTile, CTY>::NT, CTY == kFlowTY ? 2 : 3)
+__global__ void __launch_bounds__(FlowTile<CTY>::NT, CTY == kFlowTY ? 2 : 3)
     kb_collide_f32(const BatchDomain* __restrict__ doms, const int* __restrict__ map, int cur, int tcur, long long step,
                    int block0, int dom0, const __grid_constant__ FlowLaunchMaps maps) {
   const int blk = block0 + blockIdx.x, k = map[blk];
   const BatchDomain& D = doms[k];
   const int local = blk - D.coll_first;
-  flow_tile<float, kPsiDF, kFlowTile, kCollCM, CTY>(
+  flow_tile<kPsiDF, kCollCM, CTY>(
       D.g, D.ph, static_cast<const float*>(D.d.f[cur]), static_cast<float*>(D.d.f[cur ^ 1]),
       static_cast<const float*>(D.d.T[tcur]), psi_buf<float>(D, cur), D.d.mask,
       static_cast<const float*>(D.d.side[cur]), static_cast<float*>(D.d.side[cur ^ 1]), static_cast<float*>(D.d.rho),
@@ -96,7 +89,7 @@ __global__ void __launch_bounds__(EnergyTile<ETY>::NT, 960 / EnergyTile<ETY>::NT
 
 // Tensor maps of one batched domain for tile heights (cty, ety).
 inline bool batch_maps_impl_f32(BatchDomain& D, DomainMaps& m, int cty, int ety) {
-  using FT = FlowTile<float, kFlowTile, 8>;
+  using FT = FlowTile<8>;
   const Geo& g = D.g;
   bool ok = D.d.tma != 0 && static_cast<const float*>(D.d.ux) == static_cast<const float*>(D.d.rho) + g.plane &&
             static_cast<const float*>(D.d.uy) == static_cast<const float*>(D.d.rho) + 2 * (size_t)g.plane;
@@ -118,7 +111,7 @@ int batch_step_impl_f32(const BatchDomain* doms, const int* map_coll, int nb_col
     FlowLaunchMaps m;
     for (int k = d0; k < d1; ++k) m.f[k - d0] = hmaps[k].f[cur];
     const int b0 = hdoms[d0].coll_first, b1 = d1 < ndom ? hdoms[d1].coll_first : nb_coll;
-    kb_collide_f32<CTY><<<b1 - b0, FlowTile<float, kFlowTile, CTY>::NT, 0, s>>>(doms, map_coll, cur, tcur, step, b0, d0, m);
+    kb_collide_f32<CTY><<<b1 - b0, FlowTile<CTY>::NT, 0, s>>>(doms, map_coll, cur, tcur, step, b0, d0, m);
     ++n;
   }
   for (int d0 = 0; d0 < ndom; d0 += kBatchEnDomains) {
@@ -135,25 +128,25 @@ int batch_step_impl_f32(const BatchDomain* doms, const int* map_coll, int nb_col
 }  // namespace kern
 
 // ---------------------------------------------------------------- single-domain step
-template <typename S, int PSI, int MODE>
+template <int PSI>
 void launch_flow_f32(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int forcing, cudaStream_t s) {
   using namespace kern;
-  using FT = FlowTile<S, MODE, FlowRows<S, MODE>::v>;
-  const S* f = static_cast<const S*>(d.f[cur]);
+  using FT = FlowTile<kFlowTY>;
+  const float* f = static_cast<const float*>(d.f[cur]);
   CUtensorMap tm_f;
-  const bool staged = d.tma && tma::encode<S>(&tm_f, f, g.nx, g.ny, g.pitch, g.plane, 9, FT::FW, FT::FH);
+  const bool staged = d.tma && tma::encode<float>(&tm_f, f, g.nx, g.ny, g.pitch, g.plane, 9, FT::FW, FT::FH);
   const int flags = staged ? (kLaunchStaged | ((d.starve & kStarveCollide) ? kLaunchStarve : 0) |
                               ((d.pdl && d.f_ready) ? kLaunchEarlyF : 0))
                            : 0;
   const dim3 grd((g.nx + FT::TX - 1) / FT::TX, (g.ny + FT::TY - 1) / FT::TY);
   auto go = [&](auto kernel) {
-    launch_dep(d.pdl, grd, dim3(FT::NT), 0, s, kernel, g, ph, f, static_cast<S*>(d.f[cur ^ 1]),
+    launch_dep(d.pdl, grd, dim3(FT::NT), 0, s, kernel, g, ph, f, static_cast<float*>(d.f[cur ^ 1]),
                static_cast<const float*>(d.T[tcur]), static_cast<float*>(d.psi), d.mask,
                static_cast<const float*>(d.side[cur]), static_cast<float*>(d.side[cur ^ 1]), static_cast<float*>(d.rho),
                static_cast<float*>(d.ux), static_cast<float*>(d.uy), forcing, d.status, tm_f, flags);
   };
-  if (d.collision == kCollBGK) go(k_collide_f32<S, PSI, MODE, kCollBGK>);
-  else go(k_collide_f32<S, PSI, MODE, kCollCM>);
+  if (d.collision == kCollBGK) go(k_collide_f32<PSI, kCollBGK>);
+  else go(k_collide_f32<PSI, kCollCM>);
 }
 
 template <typename S, int PSI, bool PULL, int TY>
@@ -177,11 +170,14 @@ void launch_energy_f32(const Geo& g, const Phys& ph, const Dev& d, int cur, int 
              staged ? (kLaunchStaged | ((d.starve & kStarveEnergy) ? kLaunchStarve : 0)) : 0);
 }
 
-// A step takes the collision with psi in its tiles (populations stored in FP32, psi in FP32 or
-// double-float) or reads psi, which the energy pass of the step before has made (FP64 populations or
-// FP64 psi: their tiles would not fit shared memory, or cost more than the second pull) or, in a
-// first step, k_rho_psi.  On small lattices (flow_psi_in_tile) a step whose predecessor ran no energy pass
-// (a first step, a warm-up step, T fixed) takes psi from k_rho_psi too.
+// The collision of a step: with psi in its tiles (populations stored in FP32, psi in FP32 or double-float), or
+// one node per lane (launch_collide) where psi is read, or there is none: FP64 populations and FP64 psi, whose
+// tiles would not fit shared memory or cost more than a second pull, and single-phase fluids.  Pairs of columns
+// took longer there: FP64 populations 58 us against 49 at 1350 x 600 and 127 against 111 at 2048 x 1024, a single phase
+// 6.6 against 3.0 at 241 x 241, 6.3 against 4.5 at 512 x 512 and 36 against 31 at 2048 x 1024 (a step, energy pass off).
+// psi that is read comes from the energy pass of the step before or, in a first step, from k_rho_psi.  On
+// small lattices (flow_psi_in_tile) a step whose predecessor ran no energy pass (a first step, a warm-up step,
+// T fixed) takes psi from k_rho_psi too.
 template <typename S, int PSI>
 int step_impl_f32(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur, int forcing, int energy,
                   cudaStream_t s, const LaunchHook* hook, int* t_flipped, PsiChain* chain) {
@@ -207,9 +203,12 @@ int step_impl_f32(const Geo& g, const Phys& ph, const Dev& d, int cur, int tcur,
     post(kKRhoPsi);
   }
   pre(kKCollide);
-  if (!multi) launch_flow_f32<S, kPsiDF, kFlowNone>(g, ph, d, cur, tcur, forcing, s);
-  else if (!tile) launch_flow_f32<S, kPsiDF, kFlowRead>(g, ph, d, cur, tcur, forcing, s);
-  else if constexpr (can_tile) launch_flow_f32<S, PSI, kFlowTile>(g, ph, d, cur, tcur, forcing, s);
+  if constexpr (!can_tile) {
+    launch_collide<float, S>(g, ph, d, cur, forcing, nullptr, s);
+  } else {
+    if (tile) launch_flow_f32<PSI>(g, ph, d, cur, tcur, forcing, s);
+    else launch_collide<float, S>(g, ph, d, cur, forcing, nullptr, s);
+  }
   post(kKCollide);
   *t_flipped = 0;
   if (chain) chain->made = kPsiFromPass;

@@ -66,14 +66,14 @@ def _rows_gradient(at):
     return gx, gy
 
 
-@pytest.mark.parametrize("storage", ["f32", "f64", "f16s"])
+@pytest.mark.parametrize("storage,psi_mode", [("f32", 0), ("f32", 1), ("f32", 2), ("f64", 0), ("f16s", 0)])
 @pytest.mark.parametrize("nx,ny,periodic_x", [(131, 97, 0), (128, 100, 1), (61, 45, 0)])
-def test_force_planes_are_the_collisions_own(nx, ny, periodic_x, storage):
+def test_force_planes_are_the_collisions_own(nx, ny, periodic_x, storage, psi_mode):
     from paper_1912_02018_gb300 import Sim
 
     case = si.Case(nx=nx, ny=ny, D=14.0, xc=nx / 3.0, yc=ny / 2.0, Re=40.0, superheat_Tc=0.08, periodic_x=periodic_x,
                    seed=nx)
-    sim = Sim.from_case(case, f64=False, storage=storage).step(7)
+    sim = Sim.from_case(case, f64=False, storage=storage, psi_mode=psi_mode).step(7)
     got, info = sim.fields(("rho", "psi", "Fx", "Fy", "solid")), sim.info()
     sim.close()
     psi, rho = got["psi"].astype(F), got["rho"].astype(F)

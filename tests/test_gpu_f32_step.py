@@ -129,3 +129,4 @@ def test_fp32_psi_routes_and_restart(nx, ny, D, periodic_x, storage, psi_mode, c
             assert err <= 1e-5 * np.abs(ref.field(k)[fluid]).max(), (k, err)
     sim.close()
     again.close()
+
