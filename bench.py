@@ -83,8 +83,8 @@ ALG_BYTES = {
 }
 STEP_ALG_BYTES = 9 * POP * 2 + 4 * 2      # the whole step: populations and T in and out
 KERNEL_SRCS = [os.path.join(ROOT, "paper_1912_02018_gb300", "csrc", n) for n in (
-    "lbm_kernels.cuh", "lbm_tma.cuh", "lbm_step_f32.cuh", "lbm_flow_f32.cuh", "lbm_energy_f32.cuh", "lbm_energy_f64.cuh",
-    "lbm_step_f16s.cuh")]
+    "lbm_kernels.cuh", "lbm_tma.cuh", "lbm_step_f32.cuh", "lbm_flow_f32.cuh", "lbm_collide_f32.cuh", "lbm_energy_f32.cuh",
+    "lbm_energy_f64.cuh", "lbm_step_f16s.cuh")]
 
 
 def kernel_hash() -> str:

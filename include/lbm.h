@@ -34,8 +34,10 @@
  *   - lbm_step only enqueues work on the context's stream.  A fault detected by a
  *     kernel (non-finite density, non-positive psi radicand) is latched on the device
  *     and reported as LBM_EUNSTABLE by the next call that synchronises (lbm_sync,
- *     lbm_fields, lbm_get_state, lbm_wall_heat_flux); a bounded wait of a kernel that gave
- *     up is reported there as LBM_ETIMEOUT.
+ *     lbm_fields, lbm_get_state, lbm_wall_heat_flux).  The radicand of a state is checked where its
+ *     psi is evaluated: in the step that follows it (FP32 populations, T fixed, warm-up), or at
+ *     the end of the step that makes it (FP64 and FP16 storage with the energy equation).  A
+ *     bounded wait of a kernel that gave up is reported by the same calls as LBM_ETIMEOUT.
  */
 #ifndef LBM_H
 #define LBM_H

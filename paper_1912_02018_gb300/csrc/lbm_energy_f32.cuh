@@ -6,10 +6,12 @@
 // step) stay in its registers between the stages; two more warps compute stage 1 on the two halo
 // rows below and above the tile.
 //
-// Bound by instruction issue: 23.5 M warp instructions and 40 us at 2048 x 1024, against 51.9 M and 68 us
-// of 32 x 16 tiles with a lane per pair, separate stencil sums and the psi of the next step (30 M
-// and about 27 us of it).  4-row tiles where 16-row ones would leave SMs idle (12.6 us of a 192 x 96
-// lattice against 18).
+// 40 us at 2048 x 1024 for 23.7 M warp instructions.  No unit is full: 59% of the issue slots, the FMA pipe 53% of
+// the cycles (a packed operation holds it for two), DRAM 12%; three 10-warp blocks an SM (64 registers,
+// 112 B spilled) wait at the barriers (2.0 cycles an instruction), for the copies (1.8) and for the FMA pipe
+// (1.4).  32 x 16 tiles with a lane per pair, separate stencil sums and the psi of the next step took 51.9 M
+// and 68 us (30 M and about 27 us of it for that psi).  4-row tiles where 16-row ones would leave SMs idle
+// (12.6 us of a 192 x 96 lattice against 18).
 //
 // Stencils: a lane reads the 6-column window of its column pair row by row (three 8-byte loads)
 // and folds each row into sums and differences over +/-1 and +/-2 columns, from which every

@@ -7,11 +7,12 @@
 // rows too, into a shared tile.  Phase 2: the warps of the own rows take the force from the psi tile and
 // collide the moments they still hold in registers.
 //
-// Bound by the latency of a block (900 cycles of prologue, 2700 of the copy, 1600 pull, 1400 psi, 1000
-// barrier, 1500 collision, 850 stores; two blocks of 16 warps on an SM): 58 us for collision and psi
-// at 2048 x 1024, where the one-node-per-lane collision took 38 us and the psi that the energy pass
-// made for it 27 us more.  8 to 16 rows, 2 to 4 blocks and a persistent grid that prefetches the
-// next tile lie within 5% of it; 64 own columns with a wider halo take 62 us.
+// 56 us for collision and psi at 2048 x 1024, where the one-node-per-lane collision took 38 us and the psi that
+// the energy pass made for it 27 us more.  Its 32.0 M warp instructions take 53% of the issue slots, the
+// FMA pipe is busy in 37% of the cycles and DRAM in 33%: the two 16-warp blocks of an SM pass copy, pull, psi,
+// barrier, collision and stores one after the other, and there are no more warps to fill in.  8 to 16 rows, 2
+// to 4 blocks and a persistent grid that prefetches the next tile lie within 5% of it; 64 own columns with
+// a wider halo take 62 us.
 //
 // psi in the tile evaluates psi at 1.42 nodes per node, and reads each population once per step (the halo
 // comes from L2).  Collisions that read psi, or need none, run one node per lane (collide_node of

@@ -164,7 +164,7 @@ struct EnLaunchMaps {
 bool batch_maps_f32(BatchDomain& D, DomainMaps& m, int cty, int ety);
 bool batch_maps_f64(BatchDomain& D, DomainMaps& m, int cty, int ety);
 
-// FP32 collision tiles with psi: 60 x 12 nodes (48 KB of shared memory).
+// FP32 collision tiles with psi: 60 x 12 nodes (48 KB of shared memory); the others are 32 x 8.
 constexpr int kFlowTX = 60, kFlowTY = 12;
 // Tile-height variants of the batched step the autotuner chooses from: (CTY, ETY).
 constexpr int kBatchVariants = 4;
@@ -192,8 +192,8 @@ constexpr int kEnergyTX64 = 32, kEnergyTX32 = 60, kEnergyTY = 16, kEnergyTYSmall
 // Small lattices: fewer 60 x 16 energy tiles than SMs; the energy pass then takes 4-row tiles (four
 // times the blocks, each less than half as long: the pass is one wave either way).
 inline bool small_lattice(int nx, int ny) { return (long long)((nx + 59) / 60) * ((ny + 15) / 16) < 152; }
-// Lattices whose first FP32 step evaluates psi in the collision's tiles too (no psi pass at all); on
-// smaller ones that pass is 3 us of one step.
+// Lattices whose FP32 steps evaluate psi in the collision's tiles from the first one on; smaller ones run a psi
+// pass in a first step (3 us of it), which profiles of small runs count.
 inline bool flow_psi_in_tile(int nx, int ny) { return (long long)nx * ny >= 12000; }
 inline int energy_blocks(int nx, int ny) {  // upper bound over both precisions
   return ((nx + kEnergyTX64 - 1) / kEnergyTX64) * ((ny + 3) / 4);

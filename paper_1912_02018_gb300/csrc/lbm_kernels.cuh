@@ -2,10 +2,11 @@
 // templated on the compute type C (double or float) and population storage type S.
 //
 // Layout: structure of arrays, every field [ny][pitch] with x fastest; populations are
-// 9 such planes, ping-ponged between two buffers.  Here: the building blocks, and the kernels of the
-// FP64 build and of FP16 population storage (their energy passes: lbm_energy_f64.cuh, one kernel
-// per Heun stage, and lbm_step_f16s.cuh).  The FP32 step: lbm_step_f32.cuh, lbm_flow_f32.cuh,
-// lbm_energy_f32.cuh.
+// 9 such planes, ping-ponged between two buffers.  Here: the building blocks, and the collision of one node per
+// lane that the FP64 build, FP16 and FP64 population storage, FP64 psi and single-phase fluids take (the
+// energy passes of FP64 and FP16 storage: lbm_energy_f64.cuh, one kernel per Heun stage, and
+// lbm_step_f16s.cuh).  The FP32 step: lbm_step_f32.cuh, lbm_flow_f32.cuh (collision with psi in its tiles),
+// lbm_collide_f32.cuh (the arithmetic of both collisions), lbm_energy_f32.cuh.
 //   k_rho_psi pull f with boundary substitutions, rho, psi(rho, T); writes psi.  Runs only
 //             when neither an energy pass made psi nor the collision makes it (first step,
 //             after a restore, warm-up).
@@ -285,7 +286,7 @@ __device__ __forceinline__ float psi_eos_df(const Phys& ph, float rho, float T, 
   const DF r = df_sqrt(rad);
   return __fadd_rn(r.hi, r.lo);
 }
-// The same in plain FP32.
+// The same in plain FP32 (its FMA contraction is the compiler's; the tests hold its routes to equal bits).
 __device__ __forceinline__ float psi_eos_f32(const Phys& ph, float rho, float T, float& rad) {
   float s = 1.0f + ph.kappa2.hi * (1.0f - sqrtf(T * ph.invTc2.hi));
   float phi = s * s;

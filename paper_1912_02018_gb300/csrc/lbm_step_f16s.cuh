@@ -4,7 +4,7 @@
 // differ by 1e-3 within a hundred steps.  These kernels therefore keep one order of operations for good:
 // one lane per node in the collision (collide_tile of lbm_kernels.cuh, 32 x 8 tiles), a lane per
 // pair in the 32 x 16 energy tiles, whose last part makes psi of the next step.  The reordered
-// passes of lbm_flow_f32.cuh and lbm_energy_f32.cuh serve FP32 and FP64 populations only.
+// passes of lbm_flow_f32.cuh, lbm_collide_f32.cuh and lbm_energy_f32.cuh serve FP32 and FP64 populations only.
 #pragma once
 
 namespace lbm {
