@@ -399,6 +399,7 @@ lbm_status lbm_create(const lbm_domain* domain, const lbm_cylinder* cyl, const l
     const bool two = rho_l > rho_v;  // else the phase fraction is 1 everywhere
     en.T_sat = (float)T_sat;
     en.T_wall = (float)T_wall, en.th_wall = (float)(T_wall - T_sat), en.dT_sat = (float)(T_sat - en.T_sat);
+    en.dT_half = 0.5f * en.dT_sat;
     en.T_ulp = std::nextafterf(en.T_sat, INFINITY) - en.T_sat;
     en.ph1 = two ? (float)(1.0 / (rho_l - rho_v)) : 0.0f;
     en.ph0 = two ? (float)(-rho_v / (rho_l - rho_v)) : 1.0f;

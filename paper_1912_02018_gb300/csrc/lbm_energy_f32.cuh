@@ -8,7 +8,7 @@
 //
 // 40 us at 2048 x 1024 for 23.7 M warp instructions.  No unit is full: 59% of the issue slots, the FMA pipe 53% of
 // the cycles (a packed operation holds it for two), DRAM 12%; three 10-warp blocks an SM (64 registers,
-// 112 B spilled) wait at the barriers (2.0 cycles an instruction), for the copies (1.8) and for the FMA pipe
+// 124 B spilled) wait at the barriers (2.0 cycles an instruction), for the copies (1.8) and for the FMA pipe
 // (1.4).  32 x 16 tiles with a lane per pair, separate stencil sums and the psi of the next step took 51.9 M
 // and 68 us (30 M and about 27 us of it for that psi).  4-row tiles where 16-row ones would leave SMs idle
 // (12.6 us of a 192 x 96 lattice against 18).
@@ -154,15 +154,13 @@ __device__ __forceinline__ float lam_cv(const StepConst& k, float rho) {
 }
 
 // The stored temperature of theta = T - T_sat (theta_of of lbm_kernels.cuh is the way back).
-__device__ __forceinline__ float T_of(const StepConst& k, float theta) {
+__device__ __forceinline__ float2 T_of(const StepConst& k, float2 theta) {
   // the nearest temperature that can be stored.  The stored T_sat stands for theta = 0 and lies dT_sat off the
   // even spacing, so its two boundaries are dT_sat / 2 off the even ones: rounded evenly there, a bulk that
   // fluctuates about T_sat would drift by a fraction of dT_sat each step
-  const float d = fabsf(theta) < k.T_ulp ? __fmul_rn(0.5f, k.dT_sat) : k.dT_sat;
-  return __fadd_rn(k.T_sat, __fadd_rn(theta, d));
-}
-__device__ __forceinline__ float2 T_of(const StepConst& k, float2 theta) {
-  return make_float2(T_of(k, theta.x), T_of(k, theta.y));
+  const float2 d = make_float2(fabsf(theta.x) < k.T_ulp ? k.dT_half : k.dT_sat,
+                               fabsf(theta.y) < k.T_ulp ? k.dT_half : k.dT_sat);
+  return add2(f2(k.T_sat), add2(theta, d));
 }
 
 // Block-level end of the wall heat flux: one FP64 partial per tile column and 4-row group of the

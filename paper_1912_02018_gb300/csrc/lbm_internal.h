@@ -47,11 +47,11 @@ struct PhysC {
 };
 
 // Constants of the FP32 passes: phase fraction = clamp(rho ph1 + ph0).  Energy: T_sat, T_wall as
-// stored, T_wall - T_sat rounded from FP64, what the stored T_sat lacks of it, and its last place; alpha = av +
-// da times the fraction; R / c_v, a / c_v, b, b^2, 2 b of the EOS; kappa (1 + kappa) / sqrt(Tc),
-// kappa^2 / Tc.  Collision: -G / 3, sigma (G / 3)^2, and 3 nu = nv3 + dn3 times the fraction.
+// stored, T_wall - T_sat rounded from FP64, what the stored T_sat lacks of it, half of that, and its last
+// place; alpha = av + da times the fraction; R / c_v, a / c_v, b, b^2, 2 b of the EOS; kappa (1 + kappa) /
+// sqrt(Tc), kappa^2 / Tc.  Collision: -G / 3, sigma (G / 3)^2, and 3 nu = nv3 + dn3 times the fraction.
 struct StepConst {
-  float T_sat, T_wall, th_wall, dT_sat, T_ulp, ph1, ph0, da, av, rep, att, b, bb, b2, c1, c2;
+  float T_sat, T_wall, th_wall, dT_sat, dT_half, T_ulp, ph1, ph0, da, av, rep, att, b, bb, b2, c1, c2;
   float gm, sg, nv3, dn3;
 };
 
