@@ -6,7 +6,7 @@
 // step) stay in its registers between the stages; two more warps compute stage 1 on the two halo
 // rows below and above the tile.
 //
-// 40 us at 2048 x 1024 for 23.7 M warp instructions.  No unit is full: 59% of the issue slots, the FMA pipe 53% of
+// 40 us at 2048 x 1024 for 23.6 M warp instructions.  No unit is full: 59% of the issue slots, the FMA pipe 53% of
 // the cycles (a packed operation holds it for two), DRAM 12%; three 10-warp blocks an SM (64 registers,
 // 124 B spilled) wait at the barriers (2.0 cycles an instruction), for the copies (1.8) and for the FMA pipe
 // (1.4).  32 x 16 tiles with a lane per pair, separate stencil sums and the psi of the next step took 51.9 M
