@@ -130,3 +130,20 @@ def test_fp32_psi_routes_and_restart(nx, ny, D, periodic_x, storage, psi_mode, c
     sim.close()
     again.close()
 
+
+
+def test_single_phase_domain_of_a_batch():
+    # a batch collides every FP32 domain in the tiles with psi, a context of its own without psi one node per
+    # lane: the same bits
+    from paper_1912_02018_gb300 import Batch, Sim
+
+    cases = [si.Case(nx=nx, ny=ny, D=9.0, xc=nx / 3.0, yc=ny / 2.0, Re=40.0, superheat_Tc=0.05, G=G, seed=nx)
+             for nx, ny, G in ((127, 41, 0.0), (131, 97, -2.0), (64, 33, 0.0))]
+    batch = Batch(cases).step(12)
+    for i, case in enumerate(cases):
+        one = Sim.from_case(case).step(12)
+        names = ("rho", "ux", "uy", "T") + (("psi",) if case.G else ())
+        got, want = batch.domain(i).fields(names), one.fields(names)
+        for k in names:
+            assert np.array_equal(got[k], want[k]), (i, k)
+        one.close()
